@@ -112,6 +112,45 @@ __device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
+// ------------------------------------------------------------------ FP64 without the FP64 pipe's divides
+// A division or square root in FP64 is a sequence of 8 to 12 FP64 instructions, and an FP64 warp
+// instruction holds its SM partition for 64 cycles on GB300 (integer, FP32 and special-function
+// instructions: 1 to 4). The FP64 path's stepping therefore takes reciprocals and roots by
+// Newton-Raphson (or one third-order step, which cubes the relative error) from the special-function
+// unit's or an FP32 seed, and compares magnitudes as integers. Products that feed a sum are written
+// as fma() or __dmul_rn, so that every instantiation (register caps, lanes a track) rounds alike.
+
+// |x| <= lim and |x| < lim for lim >= 0: the bit patterns of non-negative doubles order like the
+// values, NaN above all (so a NaN x is neither).
+__device__ __forceinline__ bool abs_le(double x, double lim) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffll) <= __double_as_longlong(lim);
+}
+__device__ __forceinline__ bool abs_lt(double x, double lim) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffll) < __double_as_longlong(lim);
+}
+
+// 1/x of a normal x well inside the exponent range, within an ulp: the special-function seed (2^-20)
+// and one third-order step.
+__device__ __forceinline__ double rcp_nr(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// 1/sqrt(x) of a normal x > 0, within about an ulp, in the same way.
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(__dmul_rn(-x, y), y, 1.0);
+  return fma(__dmul_rn(y, e), fma(e, 0.375, 0.5), y);
+}
+
+// a . b with a fixed order of roundings
+__device__ __forceinline__ double dot3f(const double a[3], const double b[3]) {
+  return fma(a[2], b[2], fma(a[1], b[1], __dmul_rn(a[0], b[0])));
+}
+
 // ------------------------------------------------------------------ field policies
 // Uniform field along z (the solenoid axis): T x B has no z component, so T_z, and with it
 // theta, is constant along the path: the theta row of the transport Jacobian of the motion is
@@ -450,6 +489,200 @@ __device__ uint32_t propagate(const F& fld, const OptionsDev& o, const Surf& s, 
   for (int i = 0; i < 3; ++i) Bt[i] = lk * B[i];
   cross(T, Bt, kend);
   return st;
+}
+
+// ------------------------------------------------------------------ propagation, FP64, field along z
+// parabolic_path from the FP32 root of the same quadratic and two Newton steps in FP64 (relative
+// error 1e-6 -> 1e-12 -> 1e-17 while the discriminant exceeds a^2 / 4), 6 FP64 instructions instead
+// of about 30; the FP64 form near tangency and outside the FP32 range.
+__device__ __forceinline__ double parabolic_path_nr(double d, double a, double b) {
+  const float af = d2f(a), df = d2f(d), bf = d2f(b);
+  const float a2 = af * af, disc = fmaf(2.0f * bf, df, a2);
+  if (!(disc > 0.25f * a2 && fabsf(af) > 1e-6f && disc < 1e30f)) return parabolic_path(d, a, b);
+  const float sq = copysignf(sqrtf(disc), af);
+  const double inv = f2d(__fdividef(1.0f, sq)), hb = 0.5 * b;  // 1 / (a + b s) at the root
+  double s = f2d(__fdividef(2.0f * df, af + sq));
+  s = fma(-fma(s, fma(hb, s, a), -d), inv, s);
+  return fma(-fma(s, fma(hb, s, a), -d), inv, s);
+}
+
+// step_factor(tol / eps, 1/4, 4): the quarter root from FP32 and one Newton step on eps y^4 = tol
+// (relative error 1e-7 -> 1e-14), the clamped ends without FP64 work.
+__device__ __forceinline__ double step_factor_nr(double tol, float tol_f, double eps) {
+  const float qf = tol_f / d2f(eps);
+  if (!(qf > 1e-6f && qf < 1e6f)) {
+    if (qf >= 1e6f) return 4.0;
+    return step_factor(tol / eps, 0.25, 4.0);
+  }
+  const float yf = sqrtf(sqrtf(qf));
+  double y = f2d(yf);
+  const double y2 = __dmul_rn(y, y);
+  y = fma(-fma(__dmul_rn(eps, y2), y2, -tol), f2d(yf * (0.25f / tol_f)), y);
+  const double f = 0.9 * y;
+  return abs_lt(f, 0.25) ? 0.25 : (abs_lt(f, 4.0) ? f : 4.0);
+}
+
+// Adaptive RKN4 stepping as in `propagate`, for a field along z. There T x B turns the transverse
+// direction z = T_x + i T_y by -i w z (w = kappa q/p B_z) and leaves T_z alone, so that one RKN4 step
+// of length h is a multiplication by polynomials of x = h w (the discrete map itself, not the helix):
+//   z' = alpha z,  alpha = 1 - i x - x^2/2 + i x^3/6 + x^4/24
+//   (displacement)' = displacement + h beta z,  beta = 1 - i x/2 - x^2/6 + i x^3/24
+//   error estimate  h^2 |k1 - k2 - k3 + k4|_1 = |h x^3| / 4 |(x + i) z|_1,
+// and the landing's Taylor step the same with alpha = 1 - i x, beta = 1 - i x / 2. Multiplications by
+// complex numbers commute with d/dphi (a multiplication by i) and d/dtheta (a real scale), so those
+// derivative columns follow from the final state (the caller forms them); only the q/p column is
+// carried: dr, dT (x and y), with the polynomials' derivatives. The position is kept as the
+// displacement D from the start, rho = c - r_start, and `path` is the path length.
+//
+// Bound by the FP64 pipe: about 75 FP64 instructions an accepted step, against about 400 for the
+// four stages with three derivative columns (FP64 batch of 600,000 barrel + endcap tracks, tuned shape: 23.1 -> 11.9 ms).
+template <int kMode>
+__device__ uint32_t propagate_z(const FieldUniformZ& fld, const OptionsDev& o, const Surf& s, const double rho[3],
+                                double D[3], double T[3], double lam, double dr[2], double dT[2], double& path,
+                                double& h_ctrl, uint32_t& attempts, uint32_t& rejected, StepLearn& L) {
+  bool first = true;
+  uint32_t n_here = 0;
+  const double w = __dmul_rn(__dmul_rn(lam, kKappa), fld.bz), wl = kKappa * fld.bz;
+  const double d0 = dot3f(s.n, rho);
+  double d, a, b;
+  for (;;) {
+    d = d0 - dot3f(s.n, D);
+    a = dot3f(s.n, T);
+    b = __dmul_rn(w, fma(s.n[0], T[1], -__dmul_rn(s.n[1], T[0])));
+    if (abs_le(d, o.surf_tol)) break;
+    if (first) {
+      const float sl = d2f(d) / d2f(a);  // the straight-line path, in FP64 only near the limit
+      if (!(sl > -0.999f && sl < 1e30f)) {
+        const double sld = d / a;
+        if (!(sld > -1.0 && isfinite(sld))) return TKF_TRACK_SURFACE_MISSED;
+      }
+      first = false;
+    }
+    if (n_here >= o.max_steps) return TKF_TRACK_MAX_STEPS;
+    ++n_here;
+    ++attempts;
+    const double sp = parabolic_path_nr(d, a, b);
+    float xr[kMode == kRecord ? 12 : 1];
+    if constexpr (kMode == kRecord) {
+      const double r[3] = {s.c[0] - rho[0] + D[0], s.c[1] - rho[1] + D[1], s.c[2] - rho[2] + D[2]};
+      const float Tf[3] = {float(T[0]), float(T[1]), float(T[2])}, Bf[3] = {0.0f, 0.0f, fld.bzf};
+      mlp_features(s, r, Tf, lam, Bf, L.h_last, float(d / a), xr);
+    }
+    const double limit = h_ctrl;
+    const bool limited = !abs_lt(sp, limit);
+    const double h = limited ? copysign(limit, sp) : sp;
+    const double x = __dmul_rn(h, w), x2 = __dmul_rn(x, x);
+    const double eps = fabs(__dmul_rn(__dmul_rn(0.25 * h, x), x2)) * (fabs(fma(x, T[0], -T[1])) + fabs(fma(x, T[1], T[0])));
+    if (eps > o.tol) {
+      ++rejected;
+      h_ctrl = fabs(h) * step_factor_nr(o.tol, o.tol_f, eps);
+      if (h_ctrl < o.h_min) return TKF_TRACK_STEP_UNDERFLOW;
+      continue;
+    }
+    if constexpr (kMode == kRecord)  // steps the control limited: the proposals' domain
+      if (limited && eps > 0.0) put_record(L, xr, float(log(fabs(h) * sqrt(sqrt(o.tol / eps)))));
+    const double q = fma(x2, 1.0 / 24, -0.5);
+    const double al_r = fma(x2, q, 1.0), al_i = __dmul_rn(x, fma(x2, 1.0 / 6, -1.0));
+    const double be_r = fma(x2, -1.0 / 6, 1.0), be_i = __dmul_rn(x, q);
+    const double dal_i = fma(x2, 0.5, -1.0), dbe_r = x * (-1.0 / 3), dbe_i = fma(x2, 0.125, -0.5);  // d alpha: al_i + i dal_i
+    const double xl = __dmul_rn(h, wl), z0 = __dmul_rn(xl, T[0]), z1 = __dmul_rn(xl, T[1]);
+    dr[0] = fma(h, fma(-dbe_i, z1, fma(dbe_r, z0, fma(-be_i, dT[1], __dmul_rn(be_r, dT[0])))), dr[0]);
+    dr[1] = fma(h, fma(dbe_i, z0, fma(dbe_r, z1, fma(be_i, dT[0], __dmul_rn(be_r, dT[1])))), dr[1]);
+    const double m0 = fma(-dal_i, z1, fma(al_i, z0, fma(-al_i, dT[1], __dmul_rn(al_r, dT[0]))));
+    dT[1] = fma(dal_i, z0, fma(al_i, z1, fma(al_i, dT[0], __dmul_rn(al_r, dT[1]))));
+    dT[0] = m0;
+    D[0] = fma(h, fma(-be_i, T[1], __dmul_rn(be_r, T[0])), D[0]);
+    D[1] = fma(h, fma(be_i, T[0], __dmul_rn(be_r, T[1])), D[1]);
+    D[2] = fma(h, T[2], D[2]);
+    const double t0 = fma(-al_i, T[1], __dmul_rn(al_r, T[0]));
+    T[1] = fma(al_i, T[0], __dmul_rn(al_r, T[1]));
+    T[0] = t0;
+    path += h;
+    if (limited) {
+      const double fac = (eps > 0.0) ? step_factor_nr(o.tol, o.tol_f, eps) : 4.0;
+      const double hn = fabs(h) * fac;
+      h_ctrl = abs_le(hn, o.h_max) ? hn : o.h_max;
+    }
+    if constexpr (kMode == kRecord) L.h_last = float(fabs(h));
+  }
+  // the second-order Taylor step onto the plane
+  const double sp = parabolic_path_nr(d, a, b);
+  const double x = __dmul_rn(sp, w), hx = 0.5 * x;
+  const double xl = __dmul_rn(sp, wl), z0 = __dmul_rn(xl, T[0]), z1 = __dmul_rn(xl, T[1]);
+  dr[0] = fma(sp, fma(0.5, z1, fma(hx, dT[1], dT[0])), dr[0]);
+  dr[1] = fma(sp, fma(-0.5, z0, fma(-hx, dT[0], dT[1])), dr[1]);
+  const double m0 = fma(x, dT[1], dT[0]) + z1;
+  dT[1] = fma(-x, dT[0], dT[1]) - z0;
+  dT[0] = m0;
+  D[0] = fma(sp, fma(hx, T[1], T[0]), D[0]);
+  D[1] = fma(sp, fma(-hx, T[0], T[1]), D[1]);
+  D[2] = fma(sp, T[2], D[2]);
+  const double t0 = fma(x, T[1], T[0]);
+  T[1] = fma(-x, T[0], T[1]);
+  T[0] = t0;
+  path += sp;
+  return 0;
+}
+
+// Bound parameters on the target and the transport Jacobian after propagate_z, whose theta row is
+// (0, 0, 0, j33, j34): the motion keeps T_z, so only the theta and q/p columns change theta (by the
+// discrete map's drift of |T|).
+struct AxialTarget {
+  double sp2, cp2, st2, ct2;  // direction at the target
+  double nrm;                 // |T|
+  double inv_st, inv_nT, uT, vT;
+  double kphi;                // dphi of a unit path along the trajectory
+};
+
+__device__ __forceinline__ AxialTarget axial_target(const Surf& s, const double T[3], double w) {
+  AxialTarget t;
+  const double t2 = dot3f(T, T), e = t2 - 1.0;
+  // 1/|T|: the series while |T| drifted by less than 1e-6 (the tolerance keeps it far below)
+  const double inv = abs_lt(e, 1e-6) ? fma(e, fma(e, 0.375, -0.5), 1.0) : rsqrt_nr(t2);
+  t.nrm = __dmul_rn(t2, inv);
+  const double tx = __dmul_rn(T[0], inv), ty = __dmul_rn(T[1], inv);
+  t.ct2 = __dmul_rn(T[2], inv);
+  const double v = fma(ty, ty, __dmul_rn(tx, tx));
+  t.inv_st = v > 1e-200 ? rsqrt_nr(v) : 1.0 / sqrt(v);
+  t.st2 = __dmul_rn(v, t.inv_st);
+  t.cp2 = __dmul_rn(tx, t.inv_st);
+  t.sp2 = __dmul_rn(ty, t.inv_st);
+  const double a = dot3f(s.n, T);
+  t.inv_nT = abs_lt(a, 1e-200) ? 1.0 / a : rcp_nr(a);
+  t.uT = dot3f(s.u, T);
+  t.vT = dot3f(s.v, T);
+  t.kphi = -__dmul_rn(w, t.nrm);
+  return t;
+}
+
+// Rows 0..2 of one Jacobian column: the position's derivative x moved along T to the plane, and phi's
+// derivative `base` at fixed path.
+__device__ __forceinline__ void axial_column(const Surf& s, const AxialTarget& t, const double x[3], double base,
+                                             double out[3]) {
+  const double ds = __dmul_rn(-dot3f(s.n, x), t.inv_nT);
+  out[0] = fma(t.uT, ds, dot3f(s.u, x));
+  out[1] = fma(t.vT, ds, dot3f(s.v, x));
+  out[2] = fma(t.kphi, ds, base);
+}
+
+// Derivative column c (0 phi, 1 theta, 2 q/p) at the target: position's derivative and the base of
+// axial_column, from propagate_z's displacement, path and carried column; sth, cot: sin and cot of
+// theta at the start.
+__device__ __forceinline__ void axial_derivative(uint32_t c, const AxialTarget& t, const double D[3], double path,
+                                                 const double dr[2], const double dT[2], double sth, double cot,
+                                                 double x[3], double& base) {
+  const double bl = __dmul_rn(fma(-t.sp2, dT[0], __dmul_rn(t.cp2, dT[1])), t.inv_st);
+  x[0] = c == 0 ? -D[1] : (c == 1 ? __dmul_rn(cot, D[0]) : dr[0]);
+  x[1] = c == 0 ? D[0] : (c == 1 ? __dmul_rn(cot, D[1]) : dr[1]);
+  x[2] = c == 1 ? __dmul_rn(-sth, path) : 0.0;
+  base = c == 0 ? t.nrm : (c == 1 ? 0.0 : bl);
+}
+
+// j33 and j34 of the Jacobian.
+__device__ __forceinline__ void axial_theta_row(const AxialTarget& t, const double dT[2], double sth, double cot,
+                                                double& j33, double& j34) {
+  j33 = __dmul_rn(t.st2, fma(__dmul_rn(t.ct2, cot), t.nrm, sth));
+  j34 = __dmul_rn(t.ct2, fma(t.sp2, dT[1], __dmul_rn(t.cp2, dT[0])));
 }
 
 // ------------------------------------------------------------------ propagation, mixed precision
@@ -847,10 +1080,19 @@ __device__ __forceinline__ void jac_column(const R n[3], const R u[3], const R v
   out[3] = ct2 * cp2 * t[0] + ct2 * sp2 * t[1] - st2 * t[2];
 }
 
+// a0 b0 + a1 b1, rounded as the full five-term sum with zeros elsewhere
+__device__ __forceinline__ double two_terms(double a0, double b0, double a1, double b1) {
+  return fma(a1, b1, __dmul_rn(a0, b0));
+}
+__device__ __forceinline__ float two_terms(float a0, float b0, float a1, float b1) {
+  return fmaf(a1, b1, __fmul_rn(a0, b0));
+}
+
 // C <- J C J^T for the 5x5 packed symmetric C (J row 4 = e_4), over rows 0..3 of J; with kG = 4
 // lane gl computes row gl and the group exchanges the results.
-// kZ: row 3 of J is e_3 (theta conserved, a field along z): that row and column are copies.
-template <int kG, class R, bool kZ = false>
+// kZ: row 3 of J is e_3 (theta conserved, a field along z): that row and column are copies. kZ2: row 3
+// is (0, 0, 0, J33, J34) (the FP64 path in a field along z): its products have two terms.
+template <int kG, class R, bool kZ = false, bool kZ2 = false>
 __device__ __forceinline__ void transport_cov(const R J[5][5], R Cw[15], uint32_t gl, uint32_t gmask) {
   if constexpr (kG == 1) {
     R M[5][5];
@@ -861,6 +1103,12 @@ __device__ __forceinline__ void transport_cov(const R J[5][5], R Cw[15], uint32_
         if (kZ && r0 == 3) {
           M[3][c0] = Cw[S(3, c0)];
           continue;
+        }
+        if constexpr (kZ2) {
+          if (r0 == 3) {
+            M[3][c0] = two_terms(J[3][3], Cw[S(3, c0)], J[3][4], Cw[S(4, c0)]);
+            continue;
+          }
         }
         R acc = R(0);
 #pragma unroll
@@ -878,6 +1126,8 @@ __device__ __forceinline__ void transport_cov(const R J[5][5], R Cw[15], uint32_
           acc = M[r0][4];
         } else if (kZ && c0 == 3) {
           acc = M[r0][3];
+        } else if (kZ2 && c0 == 3) {
+          acc = two_terms(M[r0][3], J[3][3], M[r0][4], J[3][4]);
         } else {
           acc = R(0);
 #pragma unroll
@@ -1297,7 +1547,69 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
     }
     if (ent > 0) {
       constexpr int kCols = kG == 1 ? 3 : 1;
-      if constexpr (!kMixed) {
+      if constexpr (!kMixed && F::kAlongZ) {
+      // ---- material of the previous surface (muon hypothesis), then propagation (closed-form steps)
+      double T[3] = {__dmul_rn(sth, cph), __dmul_rn(sth, sph), cth};
+      double lam = p[4], th0sq = 0.0;
+      if (!bwd) {
+        status |= material(sp, a.mat, a.opt.mass, T, lam, th0sq);
+        if (status & kFatal) break;
+      }
+      double rho[3], D[3] = {0.0, 0.0, 0.0}, dr[2] = {0.0, 0.0}, dT[2] = {0.0, 0.0}, path = 0.0;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) rho[j] = s.c[j] - fma(p[1], sp.v[j], fma(p[0], sp.u[j], sp.c[j]));
+      status |= propagate_z<kMode == kRecord ? kRecord : kPlain>(fld, a.opt, s, rho, D, T, lam, dr, dT, path, h_ctrl,
+                                                                 attempts, rejected, learn);
+      if (status & kFatal) break;
+      // ---- bound parameters at the target and the transport Jacobian (path correction)
+      const AxialTarget t = axial_target(s, T, __dmul_rn(__dmul_rn(lam, kKappa), fld.bz));
+      sp2 = t.sp2;
+      cp2 = t.cp2;
+      st2 = t.st2;
+      ct2 = t.ct2;
+      const double inv_sth = abs_lt(sth, 1e-200) ? 1.0 / sth : rcp_nr(sth), cot = __dmul_rn(cth, inv_sth);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        double out[3];
+        axial_column(s, t, c == 0 ? sp.u : sp.v, 0.0, out);
+#pragma unroll
+        for (int rr = 0; rr < 3; ++rr) J[rr][c] = out[rr];
+      }
+      if constexpr (kG == 1) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          double x[3], base, out[3];
+          axial_derivative(uint32_t(c), t, D, path, dr, dT, sth, cot, x, base);
+          axial_column(s, t, x, base, out);
+#pragma unroll
+          for (int rr = 0; rr < 3; ++rr) J[rr][2 + c] = out[rr];
+        }
+      } else {  // this lane's derivative column (lane 3: another copy of q/p's), then exchanged
+        double x[3], base, out[3];
+        axial_derivative(gl, t, D, path, dr, dT, sth, cot, x, base);
+        axial_column(s, t, x, base, out);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+          for (int rr = 0; rr < 3; ++rr) J[rr][2 + c] = gshfl<kG>(gmask, out[rr], c);
+      }
+      J[3][0] = J[3][1] = J[3][2] = 0.0;
+      axial_theta_row(t, dT, sth, cot, J[3][3], J[3][4]);
+#pragma unroll
+      for (int c = 0; c < 5; ++c) J[4][c] = (c == 4) ? 1.0 : 0.0;
+      const double d[3] = {D[0] - rho[0], D[1] - rho[1], D[2] - rho[2]};
+      p[0] = dot3f(s.u, d);
+      p[1] = dot3f(s.v, d);
+      p[2] = 0.0;  // angles are carried as sines and cosines from here on
+      p[3] = 0.0;
+      p[4] = lam;
+      // ---- C_pred = J (C + Q) J^T, Q = diag(0, 0, th0^2/sin^2(theta), th0^2, 0)
+      if (!bwd) {
+        C[S(2, 2)] = fma(__dmul_rn(th0sq, inv_sth), inv_sth, C[S(2, 2)]);
+        C[S(3, 3)] += th0sq;
+      }
+      transport_cov<kG, double, false, true>(J, C, gl, gmask);
+      } else if constexpr (!kMixed) {
       // ---- material of the previous surface (muon hypothesis), then propagation
       double T[3] = {sth * cph, sth * sph, cth};
       double lam = p[4], th0sq = 0.0;
@@ -1489,6 +1801,12 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
           if (kMixed && F::kAlongZ && c0 == 3) {  // J row 3 is e_3 (mixed path, field along z)
             row[3] = st.P(r0, 3);
             continue;
+          }
+          if constexpr (!kMixed && F::kAlongZ) {  // J row 3 is (0, 0, 0, J33, J34)
+            if (c0 == 3) {
+              row[3] = two_terms(st.P(r0, 3), J[3][3], st.P(r0, 4), J[3][4]);
+              continue;
+            }
           }
           U acc = 0;
 #pragma unroll
