@@ -488,7 +488,7 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
     if (material_mixed(sc, a.mat, a.opt, Tm, lam, th0sq_f) & ~(TKF_TRACK_OUT_OF_FIELD)) return -1;
     th0sq = f2d(th0sq_f);
   } else {
-    if (material(sc, a.mat, a.opt.mass, T0, lam, th0sq) & ~(TKF_TRACK_OUT_OF_FIELD)) return -1;
+    if (material(sc, a.mat, a.opt, T0, lam, th0sq) & ~(TKF_TRACK_OUT_OF_FIELD)) return -1;
   }
   double x[3];
   for (int j = 0; j < 3; ++j) x[j] = sc.c[j] + br.p[0] * sc.u[j] + br.p[1] * sc.v[j];

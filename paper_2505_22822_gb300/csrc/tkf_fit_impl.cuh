@@ -150,6 +150,49 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
 __device__ __forceinline__ double dot3f(const double a[3], const double b[3]) {
   return fma(a[2], b[2], fma(a[1], b[1], __dmul_rn(a[0], b[0])));
 }
+__device__ __forceinline__ void crossf(const double a[3], const double b[3], double o[3]) {
+  o[0] = fma(a[1], b[2], -__dmul_rn(a[2], b[1]));
+  o[1] = fma(a[2], b[0], -__dmul_rn(a[0], b[2]));
+  o[2] = fma(a[0], b[1], -__dmul_rn(a[1], b[0]));
+}
+
+// Natural logarithm of a positive normal x (table-driven, after P. T. P. Tang, ACM TOMS 16, 1990):
+// x = 2^e m, c ~ 1/m from the top 7 bits of m, ln x = e ln 2 - ln c + ln(1 + z) with z = m c - 1,
+// |z| < 2^-8, by its series through z^7 (truncation below 2^-66). 11 FP64 instructions against about
+// 25 of log(); within 1.1 ulp in the callers' ranges (results of magnitude 4 to 40). Others: log().
+struct LogTable {
+  double c[128], l[128];  // c, -ln c
+};
+constexpr LogTable make_log_table() {
+  LogTable t{};
+  for (int j = 0; j < 128; ++j) {
+    const double c = 256.0 / (257.0 + 2.0 * j);
+    // -ln c = 2 artanh((1 - c) / (1 + c))
+    const double u = (1.0 - c) / (1.0 + c), u2 = u * u;
+    double sum = 0.0;
+    for (int k = 41; k >= 1; k -= 2) sum = sum * u2 + 1.0 / k;
+    t.c[j] = c;
+    t.l[j] = 2.0 * u * sum;
+  }
+  return t;
+}
+__device__ const LogTable kLogTable = make_log_table();
+
+__device__ __forceinline__ double log_nr(double x) {
+  const uint32_t hi = uint32_t(__double2hiint(x));
+  if (hi - 0x00100000u >= 0x7fe00000u) return log(x);
+  const int e = int(hi >> 20) - 1023;
+  const uint32_t j = (hi >> 13) & 127u;
+  const double m = __hiloint2double(int((hi & 0x000fffffu) | 0x3ff00000u), __double2loint(x));
+  const double z = fma(m, __ldg(&kLogTable.c[j]), -1.0);
+  double p = fma(z, 1.0 / 7, -1.0 / 6);
+  p = fma(z, p, 0.2);
+  p = fma(z, p, -0.25);
+  p = fma(z, p, 1.0 / 3);
+  p = fma(z, p, -0.5);
+  p = fma(__dmul_rn(z, z), p, z);
+  return fma(f2d(float(e)), 0.693147180559945309417, __ldg(&kLogTable.l[j])) + p;
+}
 
 // ------------------------------------------------------------------ field policies
 // Uniform field along z (the solenoid axis): T x B has no z component, so T_z, and with it
@@ -187,36 +230,59 @@ struct FieldUniform {
 struct FieldGrid {
   const float2* __restrict__ grid;
   int nr, nz;
-  double r0, z0, inv_dr, inv_dz;
+  double r0, z0, inv_dr, inv_dz, rmax, zmax;       // origin, 1/spacing, nr-1, nz-1
   float r0f, z0f, inv_drf, inv_dzf, rmaxf, zmaxf;  // FP32 copies: origin, 1/spacing, nr-1, nz-1
   static constexpr bool kUniform = false;
   static constexpr bool kAlongZ = false;
+  // FP64 instructions are the cost (see above): the radius by rsqrt_nr, range tests and the nodes'
+  // conversions on the integer pipe, the cell index from FP32 corrected to the exact one, the
+  // interpolation as three lerps a component (32 FP64 instructions against about 60; FP64 fit of
+  // 50,000 map muons, with the divisions and logarithms below: 5.56 -> 3.89 ms).
   __device__ __forceinline__ void at(const double* x, double B[3], bool& oof) const {
-    double r = sqrt(x[0] * x[0] + x[1] * x[1]);
-    double fr = (r - r0) * inv_dr;
-    double fz = (x[2] - z0) * inv_dz;
-    if (!(fr >= 0.0 && fr <= double(nr - 1) && fz >= 0.0 && fz <= double(nz - 1))) {
+    const double r2 = fma(x[1], x[1], __dmul_rn(x[0], x[0]));
+    double r, inv_r;
+    if (r2 > 1e-200) {
+      inv_r = rsqrt_nr(r2);
+      r = __dmul_rn(r2, inv_r);
+      r = fma(0.5 * inv_r, fma(-r, r, r2), r);  // exact where the root is (the map's edge decides on it)
+    } else {
+      r = sqrt(r2);
+      inv_r = r > 0.0 ? 1.0 / r : 0.0;
+    }
+    const double fr = __dmul_rn(r - r0, inv_dr), fz = __dmul_rn(x[2] - z0, inv_dz);
+    if (!(in_range(fr, rmax) && in_range(fz, zmax))) {
       B[0] = B[1] = B[2] = 0.0;
       oof = true;
       return;
     }
-    int ir = min(int(fr), nr - 2);
-    int iz = min(int(fz), nz - 2);
-    double a = fr - ir, b = fz - iz;
+    double a, b;
+    const int ir = cell(fr, nr - 2, a), iz = cell(fz, nz - 2, b);
     const float2* g = grid + size_t(iz) * nr + ir;
-    float2 g00 = __ldg(g), g01 = __ldg(g + 1), g10 = __ldg(g + nr), g11 = __ldg(g + nr + 1);
-    double w00 = (1.0 - a) * (1.0 - b), w01 = a * (1.0 - b), w10 = (1.0 - a) * b, w11 = a * b;
-    double br = w00 * g00.x + w01 * g01.x + w10 * g10.x + w11 * g11.x;
-    double bz = w00 * g00.y + w01 * g01.y + w10 * g10.y + w11 * g11.y;
-    if (r > 0.0) {
-      double s = br / r;
-      B[0] = s * x[0];
-      B[1] = s * x[1];
-    } else {
-      B[0] = 0.0;
-      B[1] = 0.0;
+    const float2 g00 = __ldg(g), g01 = __ldg(g + 1), g10 = __ldg(g + nr), g11 = __ldg(g + nr + 1);
+    const double br = lerp(b, lerp(a, f2d(g00.x), f2d(g01.x)), lerp(a, f2d(g10.x), f2d(g11.x)));
+    const double s = __dmul_rn(br, inv_r);
+    B[0] = __dmul_rn(s, x[0]);
+    B[1] = __dmul_rn(s, x[1]);
+    B[2] = lerp(b, lerp(a, f2d(g00.y), f2d(g01.y)), lerp(a, f2d(g10.y), f2d(g11.y)));
+  }
+  static __device__ __forceinline__ double lerp(double t, double lo, double hi) { return fma(t, hi - lo, lo); }
+  // 0 <= f <= top (the sign bit alone: f = -0)
+  static __device__ __forceinline__ bool in_range(double f, double top) {
+    const long long v = __double_as_longlong(f);
+    return (v >= 0 && v <= __double_as_longlong(top)) || v == (long long)(0x8000000000000000ull);
+  }
+  // min(int(f), last) of f >= 0 and the fraction f - that: FP32 rounding can be one cell off
+  static __device__ __forceinline__ int cell(double f, int last, double& frac) {
+    int i = min(int(d2f(f)), last);
+    frac = f - f2d(float(i));
+    if (__double2hiint(frac) < 0 && i > 0) {
+      --i;
+      frac = f - f2d(float(i));
+    } else if (__double2hiint(frac) >= 0x3ff00000 && i < last) {
+      ++i;
+      frac = f - f2d(float(i));
     }
-    B[2] = bz;
+    return i;
   }
   // the same interpolation in FP32 (mixed precision)
   __device__ __forceinline__ void atf(const float* x, float B[3], bool& oof) const {
@@ -275,6 +341,36 @@ __device__ __forceinline__ double parabolic_path(double d, double a, double b) {
     if (isfinite(q)) s = q;
   }
   return s;
+}
+
+// parabolic_path from the FP32 root of the same quadratic and two Newton steps in FP64 (relative
+// error 1e-6 -> 1e-12 -> 1e-17 while the discriminant exceeds a^2 / 4), 6 FP64 instructions instead
+// of about 30; the FP64 form near tangency and outside the FP32 range.
+__device__ __forceinline__ double parabolic_path_nr(double d, double a, double b) {
+  const float af = d2f(a), df = d2f(d), bf = d2f(b);
+  const float a2 = af * af, disc = fmaf(2.0f * bf, df, a2);
+  if (!(disc > 0.25f * a2 && fabsf(af) > 1e-6f && disc < 1e30f)) return parabolic_path(d, a, b);
+  const float sq = copysignf(sqrtf(disc), af);
+  const double inv = f2d(__fdividef(1.0f, sq)), hb = 0.5 * b;  // 1 / (a + b s) at the root
+  double s = f2d(__fdividef(2.0f * df, af + sq));
+  s = fma(-fma(s, fma(hb, s, a), -d), inv, s);
+  return fma(-fma(s, fma(hb, s, a), -d), inv, s);
+}
+
+// step_factor(tol / eps, 1/4, 4): the quarter root from FP32 and one Newton step on eps y^4 = tol
+// (relative error 1e-7 -> 1e-14), the clamped ends without FP64 work.
+__device__ __forceinline__ double step_factor_nr(double tol, float tol_f, double eps) {
+  const float qf = tol_f / d2f(eps);
+  if (!(qf > 1e-6f && qf < 1e6f)) {
+    if (qf >= 1e6f) return 4.0;
+    return step_factor(tol / eps, 0.25, 4.0);
+  }
+  const float yf = sqrtf(sqrtf(qf));
+  double y = f2d(yf);
+  const double y2 = __dmul_rn(y, y);
+  y = fma(-fma(__dmul_rn(eps, y2), y2, -tol), f2d(yf * (0.25f / tol_f)), y);
+  const double f = 0.9 * y;
+  return abs_lt(f, 0.25) ? 0.25 : (abs_lt(f, 4.0) ? f : 4.0);
 }
 
 // ------------------------------------------------------------------ learned step proposer
@@ -346,86 +442,95 @@ __device__ uint32_t propagate(const F& fld, const OptionsDev& o, const Surf& s, 
   uint32_t st = 0;
   bool first = true;
   uint32_t n_here = 0;
-  const double lk = lam * kKappa;
+  // per stage: e = T x kappa B (the q/p column's source), k = lam e; Bt = lam kappa B turns the columns
+  double B[3], Bk1[3], Bt1[3], e1[3], k1[3], dist, a;
+  bool oof;
   for (;;) {
-    const double dist = s.n[0] * (s.c[0] - r[0]) + s.n[1] * (s.c[1] - r[1]) + s.n[2] * (s.c[2] - r[2]);
-    const double a = dot3(s.n, T);
-    bool oof = false;
-    double B1[3], Bt1[3], k1[3];
-    fld.at(r, B1, oof);
-    for (int i = 0; i < 3; ++i) Bt1[i] = lk * B1[i];
-    cross(T, Bt1, k1);
-    if (fabs(dist) <= o.surf_tol) {
-      // second-order Taylor step onto the plane, with the derivative columns
-      if (oof) st |= TKF_TRACK_OUT_OF_FIELD;
-      const double sp = parabolic_path(dist, a, dot3(s.n, k1)), sp2 = 0.5 * sp * sp;
+    const double dc[3] = {s.c[0] - r[0], s.c[1] - r[1], s.c[2] - r[2]};
+    dist = dot3f(s.n, dc);
+    a = dot3f(s.n, T);
+    oof = false;
+    fld.at(r, B, oof);
 #pragma unroll
-      for (int c = 0; c < kCols; ++c) {
-        double q[3];
-        cross(dT[c], Bt1, q);
-        if (kCols == 1 || c == 2) {
-          double e[3], Bk[3] = {kKappa * B1[0], kKappa * B1[1], kKappa * B1[2]};
-          cross(T, Bk, e);
-          for (int i = 0; i < 3; ++i) q[i] += kCols == 1 ? qcol * e[i] : e[i];
-        }
-        for (int i = 0; i < 3; ++i) {
-          dr[c][i] += sp * dT[c][i] + sp2 * q[i];
-          dT[c][i] += sp * q[i];
-        }
-      }
-      for (int i = 0; i < 3; ++i) {
-        r[i] += sp * T[i] + sp2 * k1[i];
-        T[i] += sp * k1[i];
-      }
-      break;
+    for (int i = 0; i < 3; ++i) Bk1[i] = __dmul_rn(kKappa, B[i]);
+    crossf(T, Bk1, e1);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      Bt1[i] = __dmul_rn(lam, Bk1[i]);
+      k1[i] = __dmul_rn(lam, e1[i]);
     }
-    const double sl = dist / a;
-    if (first && !(sl > -1.0 && isfinite(sl))) return st | TKF_TRACK_SURFACE_MISSED;
-    first = false;
+    if (abs_le(dist, o.surf_tol)) break;
+    if (first) {
+      const float sl = d2f(dist) / d2f(a);  // the straight-line path, in FP64 only near the limit
+      if (!(sl > -0.999f && sl < 1e30f)) {
+        const double sld = dist / a;
+        if (!(sld > -1.0 && isfinite(sld))) return st | TKF_TRACK_SURFACE_MISSED;
+      }
+      first = false;
+    }
     if (n_here >= o.max_steps) return st | TKF_TRACK_MAX_STEPS;
     ++n_here;
     ++attempts;
-    const double sp = parabolic_path(dist, a, dot3(s.n, k1));
+    const double sp = parabolic_path_nr(dist, a, dot3f(s.n, k1));
     float x[kMode == kRecord ? 12 : 1];
     if constexpr (kMode == kRecord) {
       const float Tf[3] = {float(T[0]), float(T[1]), float(T[2])};
-      const float Bf[3] = {float(B1[0]), float(B1[1]), float(B1[2])};
-      mlp_features(s, r, Tf, lam, Bf, L.h_last, float(sl), x);
+      const float Bf[3] = {float(B[0]), float(B[1]), float(B[2])};
+      mlp_features(s, r, Tf, lam, Bf, L.h_last, float(dist / a), x);
     }
     const double limit = h_ctrl;
-    const bool limited = !(fabs(sp) < limit);
+    const bool limited = !abs_lt(sp, limit);
     const double h = limited ? copysign(limit, sp) : sp;
-    const double h2 = 0.5 * h, h6 = h * (1.0 / 6.0);
-    double B2[3], B4[3], Bt2[3], Bt4[3];
-    double k2[3], k3[3], k4[3], T2[3], T3[3], T4[3];
+    const double h2 = 0.5 * h, h6 = h * (1.0 / 6.0), hh = __dmul_rn(h, h);
+    double Bk2[3], Bk4[3], e2[3], e3[3], e4[3], k2[3], k3[3], k4[3], T2[3], T3[3], T4[3];
     if (F::kUniform) {
-      for (int i = 0; i < 3; ++i) { B2[i] = B1[i]; Bt2[i] = Bt1[i]; }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) Bk2[i] = Bk1[i];
     } else {
       double r2[3];
-      for (int i = 0; i < 3; ++i) r2[i] = r[i] + h2 * T[i] + 0.125 * h * h * k1[i];
-      fld.at(r2, B2, oof);
-      for (int i = 0; i < 3; ++i) Bt2[i] = lk * B2[i];
+      const double q8 = 0.125 * hh;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) r2[i] = fma(q8, k1[i], fma(h2, T[i], r[i]));
+      fld.at(r2, B, oof);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) Bk2[i] = __dmul_rn(kKappa, B[i]);
     }
-    for (int i = 0; i < 3; ++i) T2[i] = T[i] + h2 * k1[i];
-    cross(T2, Bt2, k2);
-    for (int i = 0; i < 3; ++i) T3[i] = T[i] + h2 * k2[i];
-    cross(T3, Bt2, k3);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) T2[i] = fma(h2, k1[i], T[i]);
+    crossf(T2, Bk2, e2);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      k2[i] = __dmul_rn(lam, e2[i]);
+      T3[i] = fma(h2, k2[i], T[i]);
+    }
+    crossf(T3, Bk2, e3);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) k3[i] = __dmul_rn(lam, e3[i]);
     if (F::kUniform) {
-      for (int i = 0; i < 3; ++i) { B4[i] = B1[i]; Bt4[i] = Bt1[i]; }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) Bk4[i] = Bk1[i];
     } else {
       double r4[3];
-      for (int i = 0; i < 3; ++i) r4[i] = r[i] + h * T[i] + 0.5 * h * h * k3[i];
-      fld.at(r4, B4, oof);
-      for (int i = 0; i < 3; ++i) Bt4[i] = lk * B4[i];
+      const double q2 = 0.5 * hh;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) r4[i] = fma(q2, k3[i], fma(h, T[i], r[i]));
+      fld.at(r4, B, oof);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) Bk4[i] = __dmul_rn(kKappa, B[i]);
     }
-    for (int i = 0; i < 3; ++i) T4[i] = T[i] + h * k3[i];
-    cross(T4, Bt4, k4);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) T4[i] = fma(h, k3[i], T[i]);
+    crossf(T4, Bk4, e4);
     double eps = 0.0;
-    for (int i = 0; i < 3; ++i) eps += fabs(k1[i] - k2[i] - k3[i] + k4[i]);
-    eps *= h * h;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      k4[i] = __dmul_rn(lam, e4[i]);
+      eps += fabs(k1[i] - k2[i] - k3[i] + k4[i]);
+    }
+    eps = __dmul_rn(eps, hh);
     if (eps > o.tol) {
       ++rejected;
-      h_ctrl = fabs(h) * step_factor(o.tol / eps, 0.25, 4.0);
+      h_ctrl = fabs(h) * step_factor_nr(o.tol, o.tol_f, eps);
       if (h_ctrl < o.h_min) return st | TKF_TRACK_STEP_UNDERFLOW;
       continue;
     }
@@ -433,95 +538,93 @@ __device__ uint32_t propagate(const F& fld, const OptionsDev& o, const Surf& s, 
     if constexpr (kMode == kRecord)  // steps the control limited: the proposals' domain
       if (limited && eps > 0.0) put_record(L, x, float(log(fabs(h) * sqrt(sqrt(o.tol / eps)))));
     // derivative columns through the accepted step (dB/dr neglected)
+    double Bt2[3], Bt4[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      Bt2[i] = F::kUniform ? Bt1[i] : __dmul_rn(lam, Bk2[i]);
+      Bt4[i] = F::kUniform ? Bt1[i] : __dmul_rn(lam, Bk4[i]);
+    }
 #pragma unroll
     for (int c = 0; c < kCols; ++c) {
-      double q1[3], q2[3], q3[3], q4[3], u2[3], u3[3], u4[3];
-      cross(dT[c], Bt1, q1);
-      if (kCols == 1 || c == 2) {
-        double e[3];
-        double Bk1[3] = {kKappa * B1[0], kKappa * B1[1], kKappa * B1[2]};
-        cross(T, Bk1, e);
-        for (int i = 0; i < 3; ++i) q1[i] += kCols == 1 ? qcol * e[i] : e[i];
-      }
-      for (int i = 0; i < 3; ++i) u2[i] = dT[c][i] + h2 * q1[i];
-      cross(u2, Bt2, q2);
-      if (kCols == 1 || c == 2) {
-        double e[3];
-        double Bk2[3] = {kKappa * B2[0], kKappa * B2[1], kKappa * B2[2]};
-        cross(T2, Bk2, e);
-        for (int i = 0; i < 3; ++i) q2[i] += kCols == 1 ? qcol * e[i] : e[i];
-      }
-      for (int i = 0; i < 3; ++i) u3[i] = dT[c][i] + h2 * q2[i];
-      cross(u3, Bt2, q3);
-      if (kCols == 1 || c == 2) {
-        double e[3];
-        double Bk2[3] = {kKappa * B2[0], kKappa * B2[1], kKappa * B2[2]};
-        cross(T3, Bk2, e);
-        for (int i = 0; i < 3; ++i) q3[i] += kCols == 1 ? qcol * e[i] : e[i];
-      }
-      for (int i = 0; i < 3; ++i) u4[i] = dT[c][i] + h * q3[i];
-      cross(u4, Bt4, q4);
-      if (kCols == 1 || c == 2) {
-        double e[3];
-        double Bk4[3] = {kKappa * B4[0], kKappa * B4[1], kKappa * B4[2]};
-        cross(T4, Bk4, e);
-        for (int i = 0; i < 3; ++i) q4[i] += kCols == 1 ? qcol * e[i] : e[i];
-      }
+      // the q/p column's source term, scaled by 0 or 1 where a lane carries one column
+      const auto source = [&](double q[3], const double e[3]) {
+        if (kCols == 1) {
+#pragma unroll
+          for (int i = 0; i < 3; ++i) q[i] = fma(qcol, e[i], q[i]);
+        } else if (c == 2) {
+#pragma unroll
+          for (int i = 0; i < 3; ++i) q[i] += e[i];
+        }
+      };
+      double q1[3], q2[3], q3[3], q4[3], u[3];
+      crossf(dT[c], Bt1, q1);
+      source(q1, e1);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i] = fma(h2, q1[i], dT[c][i]);
+      crossf(u, Bt2, q2);
+      source(q2, e2);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i] = fma(h2, q2[i], dT[c][i]);
+      crossf(u, Bt2, q3);
+      source(q3, e3);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) u[i] = fma(h, q3[i], dT[c][i]);
+      crossf(u, Bt4, q4);
+      source(q4, e4);
+#pragma unroll
       for (int i = 0; i < 3; ++i) {
-        dr[c][i] += h * dT[c][i] + h * h6 * (q1[i] + q2[i] + q3[i]);
-        dT[c][i] += h6 * (q1[i] + 2.0 * q2[i] + 2.0 * q3[i] + q4[i]);
+        const double q23 = q2[i] + q3[i], q = q1[i] + q23;
+        dr[c][i] = fma(h, fma(h6, q, dT[c][i]), dr[c][i]);
+        dT[c][i] = fma(h6, q + q23 + q4[i], dT[c][i]);
       }
     }
+#pragma unroll
     for (int i = 0; i < 3; ++i) {
-      r[i] += h * T[i] + h * h6 * (k1[i] + k2[i] + k3[i]);
-      T[i] += h6 * (k1[i] + 2.0 * k2[i] + 2.0 * k3[i] + k4[i]);
+      const double k23 = k2[i] + k3[i], k = k1[i] + k23;
+      r[i] = fma(h, fma(h6, k, T[i]), r[i]);
+      T[i] = fma(h6, k + k23 + k4[i], T[i]);
     }
     if (limited) {
-      const double fac = (eps > 0.0) ? step_factor(o.tol / eps, 0.25, 4.0) : 4.0;
-      h_ctrl = fmin(o.h_max, fabs(h) * fac);
+      const double fac = (eps > 0.0) ? step_factor_nr(o.tol, o.tol_f, eps) : 4.0;
+      const double hn = fabs(h) * fac;
+      h_ctrl = abs_le(hn, o.h_max) ? hn : o.h_max;
     }
     if constexpr (kMode == kRecord) L.h_last = float(fabs(h));
   }
-  double B[3], Bt[3];
-  bool oof = false;
+  // second-order Taylor step onto the plane, with the derivative columns
+  if (oof) st |= TKF_TRACK_OUT_OF_FIELD;
+  const double sp = parabolic_path_nr(dist, a, dot3f(s.n, k1)), sph = 0.5 * sp;
+#pragma unroll
+  for (int c = 0; c < kCols; ++c) {
+    double q[3];
+    crossf(dT[c], Bt1, q);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (kCols == 1)
+        q[i] = fma(qcol, e1[i], q[i]);
+      else if (c == 2)
+        q[i] += e1[i];
+      dr[c][i] = fma(sp, fma(sph, q[i], dT[c][i]), dr[c][i]);
+      dT[c][i] = fma(sp, q[i], dT[c][i]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    r[i] = fma(sp, fma(sph, k1[i], T[i]), r[i]);
+    T[i] = fma(sp, k1[i], T[i]);
+  }
+  oof = false;
   fld.at(r, B, oof);
   if (oof) st |= TKF_TRACK_OUT_OF_FIELD;
-  for (int i = 0; i < 3; ++i) Bt[i] = lk * B[i];
-  cross(T, Bt, kend);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) Bk1[i] = __dmul_rn(kKappa, B[i]);
+  crossf(T, Bk1, kend);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) kend[i] = __dmul_rn(lam, kend[i]);
   return st;
 }
 
 // ------------------------------------------------------------------ propagation, FP64, field along z
-// parabolic_path from the FP32 root of the same quadratic and two Newton steps in FP64 (relative
-// error 1e-6 -> 1e-12 -> 1e-17 while the discriminant exceeds a^2 / 4), 6 FP64 instructions instead
-// of about 30; the FP64 form near tangency and outside the FP32 range.
-__device__ __forceinline__ double parabolic_path_nr(double d, double a, double b) {
-  const float af = d2f(a), df = d2f(d), bf = d2f(b);
-  const float a2 = af * af, disc = fmaf(2.0f * bf, df, a2);
-  if (!(disc > 0.25f * a2 && fabsf(af) > 1e-6f && disc < 1e30f)) return parabolic_path(d, a, b);
-  const float sq = copysignf(sqrtf(disc), af);
-  const double inv = f2d(__fdividef(1.0f, sq)), hb = 0.5 * b;  // 1 / (a + b s) at the root
-  double s = f2d(__fdividef(2.0f * df, af + sq));
-  s = fma(-fma(s, fma(hb, s, a), -d), inv, s);
-  return fma(-fma(s, fma(hb, s, a), -d), inv, s);
-}
-
-// step_factor(tol / eps, 1/4, 4): the quarter root from FP32 and one Newton step on eps y^4 = tol
-// (relative error 1e-7 -> 1e-14), the clamped ends without FP64 work.
-__device__ __forceinline__ double step_factor_nr(double tol, float tol_f, double eps) {
-  const float qf = tol_f / d2f(eps);
-  if (!(qf > 1e-6f && qf < 1e6f)) {
-    if (qf >= 1e6f) return 4.0;
-    return step_factor(tol / eps, 0.25, 4.0);
-  }
-  const float yf = sqrtf(sqrtf(qf));
-  double y = f2d(yf);
-  const double y2 = __dmul_rn(y, y);
-  y = fma(-fma(__dmul_rn(eps, y2), y2, -tol), f2d(yf * (0.25f / tol_f)), y);
-  const double f = 0.9 * y;
-  return abs_lt(f, 0.25) ? 0.25 : (abs_lt(f, 4.0) ? f : 4.0);
-}
-
 // Adaptive RKN4 stepping as in `propagate`, for a field along z. There T x B turns the transverse
 // direction z = T_x + i T_y by -i w z (w = kappa q/p B_z) and leaves T_z alone, so that one RKN4 step
 // of length h is a multiplication by polynomials of x = h w (the discrete map itself, not the helix):
@@ -867,36 +970,41 @@ __device__ uint32_t propagate_mixed(const F& fld, const OptionsDev& o, const Sur
 // the Bethe bracket needs one logarithm: 1/2 ln(2 m_e W_max / I^2) - ln(hbar omega_p / I) + 1/2 - beta^2.
 // kGain: the reversed particle of the backward filter crosses the layer against the flight
 // direction and regains the mean loss (theta0 and the loss at its momentum on arrival).
+// The two logarithms, five reciprocals and roots by log_nr, rcp_nr and rsqrt_nr, the constants folded
+// on the host: about 75 FP64 instructions a layer against 210 with log() and divisions (FP64 batch of
+// 600,000 barrel + endcap tracks 11.9 -> 10.8 ms).
 template <bool kGain = false>
-__device__ __forceinline__ uint32_t material(const Surf& s, const MaterialDev& m, double mass, const double T[3],
-                                             double& lam, double& th0sq) {
+__device__ __forceinline__ uint32_t material(const Surf& s, const MaterialDev& m, const OptionsDev& o,
+                                             const double T[3], double& lam, double& th0sq) {
   th0sq = 0.0;
   if (!(s.t > 0.0)) return 0;
-  const double inv_cos = 1.0 / fabs(dot3(s.n, T));
-  const double x = s.t * inv_cos, xx0 = s.t_x0 * inv_cos;
-  const double l2 = lam * lam;
-  const double p2 = 1.0 / l2;
-  const double m2 = mass * mass;
-  const double E2 = p2 + m2, E = sqrt(E2);
-  const double inv_beta2 = 1.0 + m2 * l2;
-  const double beta2 = 1.0 / inv_beta2;
-  const double hl = 1.0 + 0.038 * log(xx0 * inv_beta2);
-  const double a = 0.0136 * E * l2;
-  th0sq = a * a * xx0 * hl * hl;
-  const double bg2 = p2 / m2;
-  const double me_m = kMe / mass;
-  const double wmax = 2.0 * kMe * bg2 / (1.0 + 2.0 * (E / mass) * me_m + me_m * me_m);
-  const double I = m.i_ev * 1e-9;
-  double bracket;
-  if (bg2 > m.bg2_density)  // density term active: ln(beta gamma) cancels
-    bracket = 0.5 * log(2.0 * kMe * wmax / (I * I)) - m.log_hwp_over_i + 0.5 - beta2;
-  else
-    bracket = 0.5 * log(2.0 * kMe * bg2 * wmax / (I * I)) - beta2;
-  const double dedx = kBetheK * m.z_over_a * inv_beta2 * bracket;
-  const double dE = dedx * m.rho * x * 1e-4;  // MeV cm^2/g * g/cm^3 * mm -> GeV
+  const double mass = o.mass, m2 = __dmul_rn(mass, mass);
+  const double l2 = __dmul_rn(lam, lam);
+  if (!abs_lt(l2, 1e300)) {  // |q/p| without a finite square: at rest, infinite scattering
+    if (kGain || isnan(l2)) return TKF_TRACK_PARTICLE_STOPPED;
+    th0sq = __longlong_as_double(0x7ff0000000000000ll);
+    lam = copysign(0.0, lam);
+    return 0;
+  }
+  const double inv_cos = rcp_nr(fabs(dot3f(s.n, T)));
+  const double x = __dmul_rn(s.t, inv_cos), xx0 = __dmul_rn(s.t_x0, inv_cos);
+  const double p2 = rcp_nr(l2);
+  const double E2 = p2 + m2, E = __dmul_rn(E2, rsqrt_nr(E2));
+  const double inv_beta2 = fma(m2, l2, 1.0);
+  const double beta2 = rcp_nr(inv_beta2);
+  const double hl = fma(0.038, log_nr(__dmul_rn(xx0, inv_beta2)), 1.0);
+  const double ah = __dmul_rn(__dmul_rn(__dmul_rn(0.0136, E), l2), hl);
+  th0sq = __dmul_rn(__dmul_rn(ah, ah), xx0);
+  const double bg2 = __dmul_rn(p2, o.inv_mass2);
+  // 2 m_e W_max / I^2 = (2 m_e / I)^2 bg2 / (1 + 2 (E/m) (m_e/m) + (m_e/m)^2)
+  const double wi = __dmul_rn(__dmul_rn(m.two_me_over_i_sq, bg2), rcp_nr(fma(E, o.two_me_over_mass2, o.one_me_mass2)));
+  // density term active: ln(beta gamma) cancels
+  const bool dense = bg2 > m.bg2_density;
+  const double bracket = fma(0.5, log_nr(dense ? wi : __dmul_rn(wi, bg2)), (dense ? 0.5 - m.log_hwp_over_i : 0.0) - beta2);
+  const double dE = __dmul_rn(__dmul_rn(__dmul_rn(m.dedx_scale, inv_beta2), bracket), x);  // GeV
   const double Ef = kGain ? E + dE : E - dE;
   if (!(Ef > mass)) return TKF_TRACK_PARTICLE_STOPPED;
-  lam = copysign(1.0 / sqrt((Ef - mass) * (Ef + mass)), lam);
+  lam = copysign(rsqrt_nr(__dmul_rn(Ef - mass, Ef + mass)), lam);
   return 0;
 }
 
@@ -940,7 +1048,11 @@ __device__ __forceinline__ uint32_t material_mixed(const Surf& s, const Material
 // sin and cos of a small angle: Taylor polynomials through x^9 / x^8 (truncation below
 // 1e-19 for |x| < 1/16), else the library sincos.
 __device__ __forceinline__ void small_sincos(double x, double& s, double& c) {
-  if (fabs(x) < 0.0625) {
+  if (abs_lt(x, 1.0 / 512)) {  // through x^5 / x^4: truncation below 2^-65
+    const double x2 = __dmul_rn(x, x);
+    s = fma(__dmul_rn(x, x2), fma(x2, 1.0 / 120, -1.0 / 6), x);
+    c = fma(x2, fma(x2, 1.0 / 24, -0.5), 1.0);
+  } else if (abs_lt(x, 0.0625)) {
     const double x2 = x * x;
     s = x * (1.0 + x2 * (-1.0 / 6 + x2 * (1.0 / 120 + x2 * (-1.0 / 5040 + x2 * (1.0 / 362880)))));
     c = 1.0 + x2 * (-0.5 + x2 * (1.0 / 24 + x2 * (-1.0 / 720 + x2 * (1.0 / 40320 - x2 * (1.0 / 3628800)))));
@@ -1166,7 +1278,9 @@ __device__ __forceinline__ void transport_cov(const R J[5][5], R Cw[15], uint32_
 // measurement of entry m: sets the gain K, the inverse residual covariance Si and the residual r,
 // updates p and C and adds r^T Si r to chi2. Returns TKF_TRACK_UPDATE_NOT_SPD (state untouched)
 // when the residual covariance is not positive definite.
-template <int kG, class U>
+// kNr (the FP64 path): the determinant's reciprocal by rcp_nr; the mixed path keeps the correctly rounded
+// division, whose last bit its FP32 copies could pass on.
+template <int kG, bool kNr, class U>
 __device__ __forceinline__ uint32_t kalman_update(const FitArgs& a, uint32_t m, double p[5], U C[15], U K[5][2],
                                                   U& Si00, U& Si01, U& Si11, U& r0, U& r1, double& chi2,
                                                   uint32_t gl, uint32_t gmask) {
@@ -1175,7 +1289,11 @@ __device__ __forceinline__ uint32_t kalman_update(const FitArgs& a, uint32_t m, 
   const U S00 = C[S(0, 0)] + V00, S01 = C[S(0, 1)] + V01, S11 = C[S(1, 1)] + V11;
   const U det = S00 * S11 - S01 * S01;
   if (!(S00 > U(0) && det > U(0))) return TKF_TRACK_UPDATE_NOT_SPD;
-  const U idet = U(1) / det;
+  U idet;
+  if constexpr (kNr)
+    idet = det > 1e-290 && det < 1e290 ? rcp_nr(det) : 1.0 / det;
+  else
+    idet = U(1) / det;
   Si00 = S11 * idet;
   Si01 = -S01 * idet;
   Si11 = S00 * idet;
@@ -1300,7 +1418,7 @@ __device__ __forceinline__ uint32_t arrival_material(const FitArgs& a, const Sur
   if constexpr (kPrec == 0) {
     const double T[3] = {st2 * cp2, st2 * sp2, ct2};
     double th0sq;
-    status = material<true>(s, a.mat, a.opt.mass, T, lam, th0sq);
+    status = material<true>(s, a.mat, a.opt, T, lam, th0sq);
     C[S(2, 2)] += th0sq / (st2 * st2);
     C[S(3, 3)] += th0sq;
   } else {
@@ -1552,7 +1670,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       double T[3] = {__dmul_rn(sth, cph), __dmul_rn(sth, sph), cth};
       double lam = p[4], th0sq = 0.0;
       if (!bwd) {
-        status |= material(sp, a.mat, a.opt.mass, T, lam, th0sq);
+        status |= material(sp, a.mat, a.opt, T, lam, th0sq);
         if (status & kFatal) break;
       }
       double rho[3], D[3] = {0.0, 0.0, 0.0}, dr[2] = {0.0, 0.0}, dT[2] = {0.0, 0.0}, path = 0.0;
@@ -1614,7 +1732,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       double T[3] = {sth * cph, sth * sph, cth};
       double lam = p[4], th0sq = 0.0;
       if (!bwd) {
-        status |= material(sp, a.mat, a.opt.mass, T, lam, th0sq);
+        status |= material(sp, a.mat, a.opt, T, lam, th0sq);
         if (status & kFatal) break;
       }
       double r[3];
@@ -1635,14 +1753,17 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
                                                                       attempts, rejected, kend, learn);
       if (status & kFatal) break;
       // ---- bound parameters at the target and the transport Jacobian (path correction)
-      const double inv_norm = 1.0 / sqrt(dot3(T, T));
+      const double t2 = dot3f(T, T), te = t2 - 1.0;
+      const double inv_norm = abs_lt(te, 1e-6) ? fma(te, fma(te, 0.375, -0.5), 1.0) : rsqrt_nr(t2);
       const double tn[3] = {T[0] * inv_norm, T[1] * inv_norm, T[2] * inv_norm};
-      st2 = sqrt(tn[0] * tn[0] + tn[1] * tn[1]);
-      const double inv_st = 1.0 / st2;
+      const double v2 = fma(tn[1], tn[1], __dmul_rn(tn[0], tn[0]));
+      const double inv_st = v2 > 1e-200 ? rsqrt_nr(v2) : 1.0 / sqrt(v2);
+      st2 = v2 * inv_st;
       ct2 = tn[2];
       cp2 = tn[0] * inv_st;
       sp2 = tn[1] * inv_st;
-      const double inv_nT = 1.0 / dot3(s.n, T);
+      const double nT = dot3f(s.n, T);
+      const double inv_nT = abs_lt(nT, 1e-200) ? 1.0 / nT : rcp_nr(nT);
 #pragma unroll
       for (int c = 0; c < 2 + kCols; ++c) {  // u, v, then this lane's derivative columns
         double x[3], t[3], out[4];
@@ -1670,7 +1791,8 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       p[4] = lam;
       // ---- C_pred = J (C + Q) J^T, Q = diag(0, 0, th0^2/sin^2(theta), th0^2, 0)
       if (!bwd) {
-        C[S(2, 2)] += th0sq / (sth * sth);
+        const double inv_sth = abs_lt(sth, 1e-200) ? 1.0 / sth : rcp_nr(sth);
+        C[S(2, 2)] = fma(__dmul_rn(th0sq, inv_sth), inv_sth, C[S(2, 2)]);
         C[S(3, 3)] += th0sq;
       }
       transport_cov<kG>(J, C, gl, gmask);
@@ -1854,7 +1976,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
     for (int j = 0; j < 5; ++j) K[j][0] = K[j][1] = U(0);
     if (measured) {
       // the track's chi2 is the forward filter's; the backward filter's goes to chi2_bwd
-      status |= kalman_update<kG>(a, m, p, C, K, Si00, Si01, Si11, r0, r1, bwd ? chi2_bwd : chi2, gl, gmask);
+      status |= kalman_update<kG, !kMixed>(a, m, p, C, K, Si00, Si01, Si11, r0, r1, bwd ? chi2_bwd : chi2, gl, gmask);
       if (status & kFatal) break;
     }  // measured
     if (!bwd && k == 0) {
@@ -2048,7 +2170,7 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
 }
 
 inline FieldGrid grid_policy(const FieldDev& f) {
-  return FieldGrid{f.grid, f.nr, f.nz, f.r0, f.z0, f.inv_dr, f.inv_dz, float(f.r0), float(f.z0), float(f.inv_dr),
+  return FieldGrid{f.grid, f.nr, f.nz, f.r0, f.z0, f.inv_dr, f.inv_dz, double(f.nr - 1), double(f.nz - 1), float(f.r0), float(f.z0), float(f.inv_dr),
                    float(f.inv_dz), float(f.nr - 1), float(f.nz - 1)};
 }
 

@@ -26,6 +26,8 @@ struct MaterialDev {
   double z_over_a, i_ev, rho, hwp_ev;
   double log_hwp_over_i;  // ln(hbar omega_p / I)
   double bg2_density;     // (beta gamma)^2 above which the density-effect term is positive
+  double two_me_over_i_sq;  // (2 m_e / I)^2
+  double dedx_scale;        // K Z/A rho 1e-4: MeV cm^2/g -> GeV per mm of path
   // FP32 copies for the mixed path
   float log_hwp_over_i_f, bg2_density_f;
   float two_me_over_i2_f;  // 2 m_e / I^2, 1/GeV
@@ -43,6 +45,7 @@ struct FieldDev {
 
 struct OptionsDev {
   double tol, h_max, h_min, surf_tol, mass;
+  double inv_mass2, two_me_over_mass2, one_me_mass2;  // 1/m^2, 2 m_e/m^2, 1 + (m_e/m)^2
   uint32_t max_steps;
   // FP32 copies for the mixed path
   float tol_f, h_max_f, h_min_f, mass_f, me_over_mass_f, surf_tol_f;
