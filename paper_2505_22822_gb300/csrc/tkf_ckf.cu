@@ -558,6 +558,51 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
       for (int j = 0; j < 15; ++j) Cp[j] = f2d(Cf[j]);
       h_ctrl = double(h);
       return m;
+    } else if constexpr (F::kAlongZ) {  // the fit's closed-form steps (propagate_z)
+      double T[3] = {T0[0], T0[1], T0[2]}, D[3] = {0.0, 0.0, 0.0}, dr[2] = {0.0, 0.0}, dT[2] = {0.0, 0.0};
+      const double rho[3] = {s.c[0] - x[0], s.c[1] - x[1], s.c[2] - x[2]};
+      double path = 0.0, h = br.h_ctrl;
+      uint32_t att = 0, rej = 0;
+      StepLearn learn{nullptr, 0, nullptr, 0.0f};
+      const uint32_t st = propagate_z<kPlain>(fld, a.opt, s, rho, D, T, lam, dr, dT, path, h, att, rej, learn);
+      const double d[3] = {D[0] - rho[0], D[1] - rho[1], D[2] - rho[2]};
+      const double l0 = dot3f(s.u, d), l1 = dot3f(s.v, d);
+      double hu, hv;
+      module_half(a, nt, uint32_t(m), hu, hv);
+      if (st || fabs(l0) > hu || fabs(l1) > hv) {
+        skip[nskip++] = uint32_t(m);
+        continue;
+      }
+      const AxialTarget t = axial_target(s, T, __dmul_rn(__dmul_rn(lam, kKappa), fld.bz));
+      const double inv_sth = abs_lt(sth, 1e-200) ? 1.0 / sth : rcp_nr(sth), cot = __dmul_rn(cth, inv_sth);
+      double J[5][5];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        double xx[3] = {c == 0 ? sc.u[0] : sc.v[0], c == 0 ? sc.u[1] : sc.v[1], c == 0 ? sc.u[2] : sc.v[2]};
+        double base = 0.0, out[3];
+        if (c >= 2) axial_derivative(uint32_t(c - 2), t, D, path, dr, dT, sth, cot, xx, base);
+        axial_column(s, t, xx, base, out);
+#pragma unroll
+        for (int rr = 0; rr < 3; ++rr) J[rr][c] = out[rr];
+        J[3][c] = 0.0;
+        J[4][c] = (c == 4) ? 1.0 : 0.0;
+      }
+      axial_theta_row(t, dT, sth, cot, J[3][3], J[3][4]);
+      pp[0] = l0;
+      pp[1] = l1;
+      pp[2] = 0.0;  // the angles as the predicted direction (increments from here on)
+      pp[3] = 0.0;
+      pdir[0] = t.sp2;
+      pdir[1] = t.cp2;
+      pdir[2] = t.st2;
+      pdir[3] = t.ct2;
+      pp[4] = lam;
+      for (int j = 0; j < 15; ++j) Cp[j] = br.C[j];
+      Cp[S(2, 2)] = fma(__dmul_rn(th0sq, inv_sth), inv_sth, Cp[S(2, 2)]);
+      Cp[S(3, 3)] += th0sq;
+      transport_cov<1, double, false, true>(J, Cp, 0u, 0xffffffffu);
+      h_ctrl = h;
+      return m;
     } else {
       double r[3] = {x[0], x[1], x[2]}, T[3] = {T0[0], T0[1], T0[2]};
       double dr[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
