@@ -727,6 +727,22 @@ __device__ uint32_t propagate_z(const FieldUniformZ& fld, const OptionsDev& o, c
   return 0;
 }
 
+// Sines and cosines of the direction T (|T| near 1), 1 / sin(theta) and |T|; 1/|T| by its series while
+// |T| drifted by less than 1e-6 (the step tolerance keeps it far below).
+__device__ __forceinline__ void bound_direction(const double T[3], double& sp, double& cp, double& st, double& ct,
+                                                double& inv_st, double& nrm) {
+  const double t2 = dot3f(T, T), e = t2 - 1.0;
+  const double inv = abs_lt(e, 1e-6) ? fma(e, fma(e, 0.375, -0.5), 1.0) : rsqrt_nr(t2);
+  nrm = __dmul_rn(t2, inv);
+  const double tx = __dmul_rn(T[0], inv), ty = __dmul_rn(T[1], inv);
+  ct = __dmul_rn(T[2], inv);
+  const double v = fma(ty, ty, __dmul_rn(tx, tx));
+  inv_st = v > 1e-200 ? rsqrt_nr(v) : 1.0 / sqrt(v);
+  st = __dmul_rn(v, inv_st);
+  cp = __dmul_rn(tx, inv_st);
+  sp = __dmul_rn(ty, inv_st);
+}
+
 // Bound parameters on the target and the transport Jacobian after propagate_z, whose theta row is
 // (0, 0, 0, j33, j34): the motion keeps T_z, so only the theta and q/p columns change theta (by the
 // discrete map's drift of |T|).
@@ -739,17 +755,7 @@ struct AxialTarget {
 
 __device__ __forceinline__ AxialTarget axial_target(const Surf& s, const double T[3], double w) {
   AxialTarget t;
-  const double t2 = dot3f(T, T), e = t2 - 1.0;
-  // 1/|T|: the series while |T| drifted by less than 1e-6 (the tolerance keeps it far below)
-  const double inv = abs_lt(e, 1e-6) ? fma(e, fma(e, 0.375, -0.5), 1.0) : rsqrt_nr(t2);
-  t.nrm = __dmul_rn(t2, inv);
-  const double tx = __dmul_rn(T[0], inv), ty = __dmul_rn(T[1], inv);
-  t.ct2 = __dmul_rn(T[2], inv);
-  const double v = fma(ty, ty, __dmul_rn(tx, tx));
-  t.inv_st = v > 1e-200 ? rsqrt_nr(v) : 1.0 / sqrt(v);
-  t.st2 = __dmul_rn(v, t.inv_st);
-  t.cp2 = __dmul_rn(tx, t.inv_st);
-  t.sp2 = __dmul_rn(ty, t.inv_st);
+  bound_direction(T, t.sp2, t.cp2, t.st2, t.ct2, t.inv_st, t.nrm);
   const double a = dot3f(s.n, T);
   t.inv_nT = abs_lt(a, 1e-200) ? 1.0 / a : rcp_nr(a);
   t.uT = dot3f(s.u, T);
@@ -1753,15 +1759,8 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
                                                                       attempts, rejected, kend, learn);
       if (status & kFatal) break;
       // ---- bound parameters at the target and the transport Jacobian (path correction)
-      const double t2 = dot3f(T, T), te = t2 - 1.0;
-      const double inv_norm = abs_lt(te, 1e-6) ? fma(te, fma(te, 0.375, -0.5), 1.0) : rsqrt_nr(t2);
-      const double tn[3] = {T[0] * inv_norm, T[1] * inv_norm, T[2] * inv_norm};
-      const double v2 = fma(tn[1], tn[1], __dmul_rn(tn[0], tn[0]));
-      const double inv_st = v2 > 1e-200 ? rsqrt_nr(v2) : 1.0 / sqrt(v2);
-      st2 = v2 * inv_st;
-      ct2 = tn[2];
-      cp2 = tn[0] * inv_st;
-      sp2 = tn[1] * inv_st;
+      double inv_st, nrm;
+      bound_direction(T, sp2, cp2, st2, ct2, inv_st, nrm);
       const double nT = dot3f(s.n, T);
       const double inv_nT = abs_lt(nT, 1e-200) ? 1.0 / nT : rcp_nr(nT);
 #pragma unroll
