@@ -231,7 +231,7 @@ namespace tkf {
 
 // Launch policy (tkf_policy.cu). The block shape of a call: the explicit one of the options,
 // the context's tuned one for the launch class (timing the candidates on the first call when
-// TKF_FIT_AUTOTUNE is set), else the default.
+// TKF_FIT_AUTOTUNE is set), else the one for the batch's size.
 bool valid_block_shape(uint32_t threads, uint32_t blocks_per_sm, uint32_t tracks_per_warp, uint32_t max_registers,
                        uint32_t lanes_per_track, int precision, bool record);
 cudaError_t resolve_shape(tkf_context_s* ctx, const FitArgs& a, const FieldDev& f, int precision, const Workspace& ws,
@@ -242,7 +242,7 @@ cudaError_t launch_with_policy(tkf_context_s* ctx, const FitArgs& a, const Field
                                const Workspace& ws, LaunchShape shape, bool use_graph, cudaStream_t stream,
                                const cudaEvent_t* timing);
 void load_tune_cache(tkf_context_s* ctx);
-// The launch shape used without tuning or explicit options.
+// The fixed default shape (the base of partly explicit options), whatever the batch's size.
 LaunchShape default_launch_shape(int precision, bool record, int sm_count);
 void release_graph(tkf_context_s* ctx);
 

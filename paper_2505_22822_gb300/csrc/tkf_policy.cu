@@ -39,12 +39,46 @@ constexpr int kTracksPerWarp[] = {32, 16, 8, 4};
 constexpr int kGroupTracksPerWarp[] = {8, 4, 2, 1};
 constexpr int kResidentWarpsPerSm = 8;
 
-// Defaults without tuning: FP64 128 x 2 at 255 registers; mixed 128 x 4 at 128 registers (the
-// best single shape over the uniform-field and field-map batches); record capture keeps the
-// full register file (its kernels exist only there).
+// Fixed defaults, the base of partly explicit options: FP64 128 x 2 at 255 registers; mixed 128 x 4 at
+// 128 registers (the best single shape over the uniform-field and field-map batches); record
+// capture keeps the full register file (its kernels exist only there).
 std::array<int, 5> default_shape(int precision, bool record) {
   if (precision == TKF_MIXED && !record) return {128, 4, 32, 128, 1};
   return {128, 2, 32, 255, 1};
+}
+
+// Launch shape without tuning of the FP64 and mixed paths by the batch's size (record capture and explicit
+// options keep the fixed defaults). Sizes are in lanes of the full-register kernels (8 warps an SM: 38,912
+// on 152 SMs); both sides of each line measured on barrel + endcap tracks (uniform field / map), ms:
+// * RTS below 80 tracks an SM (12,160; a wave of four-lane groups is 64 an SM): four lanes a track, the
+//   warps' tracks halved while every SM still gets a warp. FP64 3,000 tracks 0.87 -> 0.55 / 2.96 -> 2.31,
+//   12,500 1.03 -> 0.78 / 3.52 -> 2.60; mixed 3,000 0.36 -> 0.31 / 0.65 -> 0.44, 12,500 0.40 -> 0.40 /
+//   0.63 -> 0.61; at 20,000 one lane wins (mixed 0.46 against 0.55 / 0.65 against 0.88).
+// * mixed: the full register file while few warps are resident anyway (latency bound: no spills), up to 1.75
+//   waves (60,000 0.77 -> 0.68 / 1.06 -> 0.96; 80,000 0.86 against 0.90 / 1.14 against 1.23), then 128
+//   registers, and 64 once their 32 warps an SM are filled several times: RTS from 6 waves (200,000 1.94
+//   against 1.97 / 2.58 against 2.44; 300,000 2.87 -> 2.77 / 3.75 -> 3.43), two-filter from 3.5 (100,000
+//   1.72 against 1.95 / 2.59 against 2.75; 150,000 2.58 -> 2.36 / 3.74 -> 3.42). The all-states mode, which
+//   stores every entry, keeps the full register file (128: 100,000 tracks with holes 2.48 against 2.54).
+// * FP64: the full register file (within 3 % of the best at every size: the FP64 pipe is the bottleneck).
+// * blocks of one warp, no more than there are chunks of tracks, while they are fewer than the resident
+//   warps: the block scheduler then spreads them evenly over the SMs (two-filter FP64 10,000 1.48 -> 1.28).
+LaunchShape sized_shape(const FitArgs& a, int precision, uint32_t sms) {
+  const uint32_t n = a.n_tracks, wave = 32 * kResidentWarpsPerSm * sms;
+  const bool two_filter = a.smoother == TKF_SMOOTHER_TWO_FILTER, states = a.states_par != nullptr;
+  LaunchShape s;
+  if (!two_filter && !states && n <= 80 * sms) {
+    s.group = 4;
+    s.tracks_per_warp = 8;
+    while (s.tracks_per_warp > 1 && n <= uint32_t(s.tracks_per_warp / 2) * sms) s.tracks_per_warp /= 2;
+  } else if (precision == TKF_MIXED && !states && n > wave / 4 * 7) {
+    s.regs = n > (two_filter ? wave / 2 * 7 : wave * 6) ? 64 : 128;
+  }
+  const uint32_t chunks = (n + s.tracks_per_warp - 1) / s.tracks_per_warp;
+  const uint32_t per_sm = s.regs == 255 ? kResidentWarpsPerSm : 65536 / (s.regs * 32);  // warps
+  s.threads = chunks < per_sm * sms ? 32 : 128;
+  s.blocks = int(s.threads == 32 ? chunks : per_sm / 4 * sms);
+  return s;
 }
 
 // Lanes a track the kernels of a precision and mode exist with.
@@ -300,6 +334,8 @@ cudaError_t resolve_shape(tkf_context ctx, const FitArgs& a, const FieldDev& f, 
       out->blocks = (65536 / (out->regs * 128)) * ctx->sm_count;
   }
   const bool any_explicit = explicit_block || o->tracks_per_warp || o->max_registers || o->lanes_per_track;
+  if (!any_explicit && !a.records && (precision == TKF_FP64 || precision == TKF_MIXED))
+    *out = sized_shape(a, precision, uint32_t(ctx->sm_count > 0 ? ctx->sm_count : 1));
   if (any_explicit || !(o->flags & TKF_FIT_AUTOTUNE) || a.records) return cudaSuccess;
   const std::string key = tune_key(a, f, precision, ctx->sm_count);
   auto it = ctx->tuned.find(key);
