@@ -2,15 +2,17 @@
 //
 // Network: 12 inputs -> 64 SiLU -> 64 SiLU -> 1, parameters packed as W1 [64][12], b1 [64],
 // W2 [64][64], b2 [64], w3 [64], b3 (FP32 master copy). Loss: mean squared error. Optimiser:
-// Adam (Kingma & Ba 2015). One training step on a batch of B samples is two launches:
-//   mlp_train_tc_kernel: one CTA per 128 samples; the forward and backward pass with every
+// Adam (Kingma & Ba 2015). A training step on a batch of B samples is
+//   the tiles (train_tile): one CTA per 128 samples; the forward and backward pass with every
 //     dense contraction on the tensor cores (tcgen05.mma kind::f16, BF16 operands, FP32
 //     accumulation in tensor memory): the two layers, the backpropagation through layer 2, and
 //     the weight gradients of both layers together with the bias gradients (one M128 N96 K128
 //     product per CTA); the output layer, bias, SiLU and its derivative on the CUDA cores in
 //     FP32; each CTA writes its partial gradient;
-//   mlp_reduce_adam_kernel: one thread per parameter; the partials summed in CTA order (no
-//     atomics: deterministic), then the Adam step.
+//   then the partials summed in CTA order (no atomics: deterministic) and the Adam step.
+// mlp_train_steps_kernel runs up to 256 steps in one cooperative launch; mlp_train_tc_kernel and
+// mlp_reduce_adam_kernel are one step in two launches (the gradient alone, and devices whose SMs
+// cannot hold a batch's CTAs at once).
 // Around training: seeded initialisation, calibration of the output bias (a quantile of the
 // training residuals, by a radix select on the device) and rounding to the BF16 weights the
 // fit's inference uses.
@@ -75,10 +77,11 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const float* __restric
 }
 
 // ---- training on the tensor cores
-// One CTA of 128 threads per tile of 128 samples, thread s = sample s = accumulator row s.
-// Operands in shared memory are K-major, no swizzle, 8 x 16-byte core matrices (core_offset);
-// a K16 step of an operand with g groups of 8 along K starts 256 bytes further, its K groups
-// are 128 bytes apart and its row groups g x 128 bytes apart.
+// One CTA of 512 threads per tile of 128 samples. Sample s is accumulator row s; four threads share a
+// sample (warps w, w + 4, w + 8, w + 12 read the same 32 tensor-memory lanes), each takes a quarter of
+// the columns. Operands in shared memory are K-major, no swizzle, 8 x 16-byte core matrices
+// (core_offset); a K16 step of an operand with g groups of 8 along K starts 256 bytes further, its K
+// groups are 128 bytes apart and its row groups g x 128 bytes apart.
 //   xa  [128 x 16]   features (12, then zeros)           layer 1:  Z1 = X W1^T       M128 N64 K16
 //   a1  [128 x 64]   SiLU(Z1 + b1)                        layer 2:  Z2 = A1 W2^T      M128 N64 K64
 //   dz2 [128 x 64]   dL/dZ2 = dout w3 SiLU'(Z2 + b2)      back:     dA1 = dZ2 W2      M128 N64 K64
@@ -89,7 +92,14 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const float* __restric
 // w3 and b3 get their gradients on the CUDA cores (FP32, a fixed-order sum over the tile).
 // BF16 operands are rounded to nearest even from the FP32 values; the products are exact and
 // summed in FP32.
+//
+// A step's work is tiny (8 tiles at batch 1024) and serial: it is bound by latencies, not by the
+// tensor cores. With one thread a sample and two launches a step it took 42 us (a 32-way bank
+// conflict in the tile's sums alone 4 us); four threads a sample, padded sums that overlap the last
+// product, and many steps a launch (mlp_train_steps_kernel) bring it to 17 us
+// (two epochs of 380,000 records: 31.7 -> 12.9 ms, the same bits).
 constexpr int kTile = 128;
+constexpr int kTrainThreads = 512;
 constexpr uint32_t kIdescN64 = umma_idesc_bf16(128, 64);
 constexpr uint32_t kIdescN96 = umma_idesc_bf16(128, 96);
 static_assert(kIdescN64 == kIdescM128N64, "instruction descriptor");
@@ -103,189 +113,309 @@ struct __align__(1024) TrainSmem {
   uint8_t w2t[64 * 64 * 2];   // W2^T (N = i, K = j)
   uint8_t xa[128 * 16 * 2];
   uint8_t w1[64 * 16 * 2];    // W1 (N = j, K = inputs, 12..15 zero)
-  float red[66][kTile];       // per-sample dout a2[j] (j < 64), dout, squared residual
+  float red[66][kTile + 1];   // per-sample a2[j], then dout a2[j] (j < 64), dout, squared residual; padded
   float b1[64], b2[64], w3[64], b3;
   uint64_t mbar;
-  uint32_t tmem_base;
+  uint32_t tmem_base, flag;
 };
 
 __device__ __forceinline__ void st_bf16(uint8_t* base, uint32_t off, float v) {
   *reinterpret_cast<uint16_t*>(base + off) = uint16_t(bf16_rne(v));
 }
 
-// Issues `nk` K16 steps of D = A B^T into tensor memory (thread 0), commits them to the
-// mbarrier and waits (every thread, bounded). Returns false if the wait ran out.
-__device__ bool tc_stage(TrainSmem& sm, uint32_t tmem, const uint8_t* a, uint32_t a_sbo, const uint8_t* b,
-                         uint32_t b_sbo, int nk, uint32_t idesc, uint32_t& phase, bool stall) {
+// 16 / 8 consecutive FP32 accumulator columns of this thread's row of tensor memory.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = __uint_as_float(r[k]);
+}
+
+// mbar_wait that polls without sleeping first: a product of this size takes a few hundred cycles.
+__device__ __forceinline__ bool mbar_poll(uint64_t* mbar, uint32_t parity) {
+  for (uint32_t it = 0; it < 4096; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(smem_addr(mbar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return mbar_wait(mbar, parity);
+}
+
+// Issues `nk` K16 steps of D = A B^T into tensor memory (thread 0) after every thread's operand stores,
+// and commits them to the mbarrier.
+__device__ void tc_issue(TrainSmem& sm, uint32_t tmem, const uint8_t* a, uint32_t a_sbo, const uint8_t* b,
+                         uint32_t b_sbo, int nk, uint32_t idesc) {
   fence_async_smem();
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && !stall) {
+  if (threadIdx.x == 0) {
     tc_fence_after();
     for (int k = 0; k < nk; ++k)
       tc_mma_id(tmem, umma_desc(smem_addr(a) + k * 256, 128, a_sbo), umma_desc(smem_addr(b) + k * 256, 128, b_sbo),
                 idesc, k > 0 ? 1u : 0u);
     tc_commit(&sm.mbar);
   }
-  const bool done = mbar_wait(&sm.mbar, phase);
+}
+// Waits for it (every thread, bounded). Returns false, in every thread, if a wait ran out.
+__device__ bool tc_await(TrainSmem& sm, uint32_t& phase) {
+  const bool done = mbar_poll(&sm.mbar, phase);
   phase ^= 1u;
   __syncwarp();
   tc_fence_after();
   return __syncthreads_or(!done) == 0;
 }
 
-// Forward and backward pass of one tile; the CTA's partial gradient (TKF_MLP_PARAMS floats) and
-// its sum of squared residuals go to part[blockIdx.x] and sq[blockIdx.x]. `inv_n`: 1 / batch
-// size (dL/dout = 2 r / n). A wait that ran out leaves NaN partials (and so NaN losses).
-__global__ void __launch_bounds__(kTile, 1) mlp_train_tc_kernel(const float* __restrict__ p, const float* __restrict__ x,
-                                                                 int x_stride, const float* __restrict__ y, int y_stride,
-                                                                 uint32_t n, float inv_n, float* __restrict__ part,
-                                                                 float* __restrict__ sq) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  // the operands at a 1024-byte boundary (the launch reserves the slack)
-  const uint32_t pad = (1024u - (smem_addr(smem_raw) & 1023u)) & 1023u;
-  TrainSmem& sm = *reinterpret_cast<TrainSmem*>(smem_raw + pad);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  // weights as BF16 operands (both orientations of W2), biases and w3 in FP32
-  for (int e = tid; e < 64 * 16; e += kTile) {
-    const int j = e >> 4, i = e & 15;
-    st_bf16(sm.w1, core_offset(j, i, 2), i < kIn ? p[oW1 + j * kIn + i] : 0.0f);
-  }
-  for (int e = tid; e < 64 * 64; e += kTile) {
-    const int j = e >> 6, i = e & 63;
-    const float w = p[oW2 + e];
-    st_bf16(sm.w2, core_offset(j, i, 8), w);
-    st_bf16(sm.w2t, core_offset(i, j, 8), w);
-  }
-  if (tid < 64) {
-    sm.b1[tid] = p[oB1 + tid];
-    sm.b2[tid] = p[oB2 + tid];
-    sm.w3[tid] = p[oW3 + tid];
-  }
+// A value of row `j` (even) and of row j + 1 at K = this thread's sample, into an operand with 16 K
+// groups: lane pairs (consecutive samples) exchange one value each, so that a lane stores one 32-bit
+// word of one row.
+__device__ __forceinline__ void st_bf16_pair(uint8_t* base, int j, int s, float v0, float v1) {
+  const uint32_t lane = threadIdx.x & 31u, odd = lane & 1u;
+  const uint32_t b0 = bf16_rne(v0), b1 = bf16_rne(v1);
+  const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? b0 : b1, 1);
+  const uint32_t word = odd ? (got | (b1 << 16)) : (b0 | (got << 16));
+  *reinterpret_cast<uint32_t*>(base + core_offset(j + int(odd), s & ~1, 16)) = word;
+}
+
+// 8 consecutive K values of one row of an operand (one 16-byte store)
+__device__ __forceinline__ void st_bf16x8(uint8_t* at, const float* v) {
+  uint32_t w[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) w[q] = bf16_rne(v[2 * q]) | (bf16_rne(v[2 * q + 1]) << 16);
+  *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// One CTA's set-up: mbarrier, 128 accumulator columns (each stage writes from column 0), the operands'
+// constant rows. Returns the tensor-memory base.
+__device__ uint32_t train_setup(TrainSmem& sm) {
+  const int tid = threadIdx.x;
   if (tid == 0) {
-    sm.b3 = p[oB3];
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sm.mbar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {  // 128 accumulator columns: each stage writes from column 0
+  if (tid < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_addr(&sm.tmem_base))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  // this sample's inputs (rows beyond the batch: zeros, and no gradient)
-  const uint32_t s = blockIdx.x * kTile + tid;
-  const bool live = s < n;
-  float xv[kIn], yv = 0.0f;
-  for (int i = 0; i < kIn; ++i) xv[i] = live ? x[size_t(s) * x_stride + i] : 0.0f;
-  if (live) yv = y[size_t(s) * y_stride];
-  for (int i = 0; i < 16; ++i) {
-    const float v = i < kIn ? xv[i] : 0.0f;
-    st_bf16(sm.xa, core_offset(tid, i, 2), v);
-    st_bf16(sm.bg, core_offset(64 + i, tid, 16), v);  // X^T
-  }
-  st_bf16(sm.bg, core_offset(80, tid, 16), 1.0f);  // ones: the bias gradients
-  for (int r = 81; r < 96; ++r) st_bf16(sm.bg, core_offset(r, tid, 16), 0.0f);
-  fence_async_smem();
+  for (int e = tid; e < 16 * kTile; e += kTrainThreads)  // the ones (bias gradients) and the zeros below
+    st_bf16(sm.bg, core_offset(80 + e / kTile, e % kTile, 16), e < kTile ? 1.0f : 0.0f);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
-  const uint32_t t_row = tmem + (uint32_t(warp * 32) << 16);  // this warp's 32 lanes
-  uint32_t phase = 0;
-  bool ok = true;
-  float v[32], d1[64];  // d1: SiLU'(Z1 + b1) of this sample
-  // layer 1
-  ok = tc_stage(sm, tmem, sm.xa, 256, sm.w1, 256, 1, kIdescN64, phase, false);
-  if (ok) {
-    for (int half = 0; half < 2; ++half) {
-      tmem_ld32(t_row + uint32_t(half * 32), v);
-      for (int k = 0; k < 32; ++k) {
-        const int j = half * 32 + k;
-        const float z = v[k] + sm.b1[j], sg = sigm(z), a = z * sg;
-        d1[j] = sg * (1.0f + z * (1.0f - sg));
-        st_bf16(sm.a1, core_offset(tid, j, 8), a);
-        st_bf16(sm.bg, core_offset(j, tid, 16), a);  // A1^T
-      }
-    }
-    // layer 2
-    ok = tc_stage(sm, tmem, sm.a1, 1024, sm.w2, 1024, 4, kIdescN64, phase, false);
-  }
-  if (ok) {
-    float z2[64], a2[64];
-    float out = sm.b3;
-    for (int half = 0; half < 2; ++half) {
-      tmem_ld32(t_row + uint32_t(half * 32), v);
-      for (int k = 0; k < 32; ++k) {
-        const int j = half * 32 + k;
-        z2[j] = v[k] + sm.b2[j];
-        a2[j] = z2[j] * sigm(z2[j]);
-        out = fmaf(sm.w3[j], a2[j], out);
-      }
-    }
-    const float r = live ? out - yv : 0.0f;
-    const float dout = 2.0f * r * inv_n;
-    for (int j = 0; j < 64; ++j) {
-      const float sg = sigm(z2[j]);
-      const float dz = dout * sm.w3[j] * (sg * (1.0f + z2[j] * (1.0f - sg)));
-      st_bf16(sm.dz2, core_offset(tid, j, 8), dz);
-      st_bf16(sm.ag, core_offset(j, tid, 16), dz);  // dZ2^T
-      sm.red[j][tid] = dout * a2[j];
-    }
-    sm.red[64][tid] = dout;
-    sm.red[65][tid] = r * r;
-    // backpropagation through layer 2
-    ok = tc_stage(sm, tmem, sm.dz2, 1024, sm.w2t, 1024, 4, kIdescN64, phase, false);
-  }
-  if (ok) {
-    for (int half = 0; half < 2; ++half) {
-      tmem_ld32(t_row + uint32_t(half * 32), v);
-      for (int k = 0; k < 32; ++k) {
-        const int i = half * 32 + k;
-        st_bf16(sm.ag, core_offset(64 + i, tid, 16), v[k] * d1[i]);  // dZ1^T
-      }
-    }
-    // weight and bias gradients of both layers: G = ag bg^T over the tile's samples
-    ok = tc_stage(sm, tmem, sm.ag, 2048, sm.bg, 2048, 8, kIdescN96, phase, false);
-  }
-  float* g = part + size_t(blockIdx.x) * kMlpParams;
-  const float nan = __int_as_float(0x7fc00000);
-  if (ok) {
-    // row tid of G: dW2 row tid and db2 (tid < 64), or dW1 row tid - 64 and db1
-    for (int c = 0; c < 3; ++c) {
-      tmem_ld32(t_row + uint32_t(c * 32), v);
-      for (int k = 0; k < 32; ++k) {
-        const int col = c * 32 + k;
-        if (tid < 64) {
-          if (col < 64) g[oW2 + tid * 64 + col] = v[k];
-          if (col == 80) g[oB2 + tid] = v[k];
-        } else {
-          if (col >= 64 && col < 64 + kIn) g[oW1 + (tid - 64) * kIn + (col - 64)] = v[k];
-          if (col == 80) g[oB1 + tid - 64] = v[k];
-        }
-      }
-    }
-    // w3, b3 and the squared residuals: sums over the tile in sample order
-    if (tid < 66) {
-      float acc = 0.0f;
-      for (int t = 0; t < kTile; ++t) acc += sm.red[tid][t];
-      if (tid < 64)
-        g[oW3 + tid] = acc;
-      else if (tid == 64)
-        g[oB3] = acc;
-      else
-        sq[blockIdx.x] = acc;
-    }
-  } else {
-    for (int k = tid; k < kMlpParams; k += kTile) g[k] = nan;
-    if (tid == 0) sq[blockIdx.x] = nan;
-    mbar_wait(&sm.mbar, phase ^ 1u);  // give an MMA still in flight a bounded time to finish
-  }
+  return sm.tmem_base;
+}
+__device__ void train_teardown(uint32_t tmem) {
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (threadIdx.x < 32) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem) : "memory");
   }
+}
+
+// Parameters as BF16 operands (both orientations of W2), biases and w3 in FP32. The loads skip L1: the
+// parameters change between the steps of one launch.
+__device__ void train_weights(TrainSmem& sm, const float* __restrict__ p) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int q = 0; q < 64 * 16 / kTrainThreads; ++q) {
+    const int e = tid + q * kTrainThreads, j = e >> 4, i = e & 15;
+    st_bf16(sm.w1, core_offset(j, i, 2), i < kIn ? __ldcg(p + oW1 + j * kIn + i) : 0.0f);
+  }
+  float w[64 * 64 / kTrainThreads];
+#pragma unroll
+  for (int q = 0; q < 64 * 64 / kTrainThreads; ++q) w[q] = __ldcg(p + oW2 + tid + q * kTrainThreads);
+#pragma unroll
+  for (int q = 0; q < 64 * 64 / kTrainThreads; ++q) {
+    const int e = tid + q * kTrainThreads, j = e >> 6, i = e & 63;
+    st_bf16(sm.w2, core_offset(j, i, 8), w[q]);
+    st_bf16(sm.w2t, core_offset(i, j, 8), w[q]);
+  }
+  if (tid < 64)
+    sm.b1[tid] = __ldcg(p + oB1 + tid);
+  else if (tid < 128)
+    sm.b2[tid - 64] = __ldcg(p + oB2 + tid - 64);
+  else if (tid < 192)
+    sm.w3[tid - 128] = __ldcg(p + oW3 + tid - 128);
+  else if (tid == 192)
+    sm.b3 = __ldcg(p + oB3);
+}
+
+// This thread's quarter of its sample's inputs (4 of 16, the last four zero) and the label.
+struct TrainInput {
+  float x[4], y;
+};
+__device__ __forceinline__ TrainInput train_input(const float* __restrict__ x, int x_stride,
+                                                  const float* __restrict__ y, int y_stride, uint32_t n) {
+  const uint32_t s = blockIdx.x * kTile + (threadIdx.x & (kTile - 1)), cg = threadIdx.x >> 7;
+  TrainInput in{{0.0f, 0.0f, 0.0f, 0.0f}, 0.0f};
+  if (s < n) {
+    if (cg < kIn / 4)
+      for (int i = 0; i < 4; ++i) in.x[i] = x[size_t(s) * x_stride + cg * 4 + i];
+    in.y = y[size_t(s) * y_stride];
+  }
+  return in;
+}
+
+// Forward and backward pass of one tile; the CTA's partial gradient (TKF_MLP_PARAMS floats) and
+// its sum of squared residuals go to g and *sq. `inv_n`: 1 / batch size (dL/dout = 2 r / n). Returns
+// false (nothing written) if a wait for the tensor cores ran out.
+__device__ bool train_tile(TrainSmem& sm, uint32_t tmem, uint32_t& phase, const TrainInput& in, uint32_t n, float inv_n,
+                           float* __restrict__ g, float* __restrict__ sq) {
+  const int tid = threadIdx.x, s = tid & (kTile - 1), cg = tid >> 7, c0 = cg * 16;
+  const bool live = blockIdx.x * kTile + s < n;
+  const uint32_t t_row = tmem + (uint32_t(s & ~31) << 16);  // this warp's 32 lanes
+  for (int i = 0; i < 4; i += 2) {
+    st_bf16(sm.xa, core_offset(s, cg * 4 + i, 2), in.x[i]);
+    st_bf16(sm.xa, core_offset(s, cg * 4 + i + 1, 2), in.x[i + 1]);
+    st_bf16_pair(sm.bg, 64 + cg * 4 + i, s, in.x[i], in.x[i + 1]);  // X^T
+  }
+  float v[16], d1[16], z2[16], sg2[16];  // d1: SiLU'(Z1 + b1)
+  // layer 1
+  tc_issue(sm, tmem, sm.xa, 256, sm.w1, 256, 1, kIdescN64);
+  if (!tc_await(sm, phase)) return false;
+  tmem_ld16(t_row + uint32_t(c0), v);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const float z = v[k] + sm.b1[c0 + k], sg = sigm(z);
+    v[k] = z * sg;
+    d1[k] = sg * (1.0f + z * (1.0f - sg));
+  }
+#pragma unroll
+  for (int k = 0; k < 16; k += 8) st_bf16x8(sm.a1 + core_offset(s, c0 + k, 8), v + k);
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.bg, c0 + k, s, v[k], v[k + 1]);  // A1^T
+  // layer 2
+  tc_issue(sm, tmem, sm.a1, 1024, sm.w2, 1024, 4, kIdescN64);
+  if (!tc_await(sm, phase)) return false;
+  tmem_ld16(t_row + uint32_t(c0), v);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    z2[k] = v[k] + sm.b2[c0 + k];
+    sg2[k] = sigm(z2[k]);
+    v[k] = z2[k] * sg2[k];
+    sm.red[c0 + k][s] = v[k];
+  }
+  __syncthreads();
+  if (cg == 0) {  // the output layer, in column order
+    float out = sm.b3;
+#pragma unroll 16
+    for (int j = 0; j < 64; ++j) out = fmaf(sm.w3[j], sm.red[j][s], out);
+    const float r = live ? out - in.y : 0.0f;
+    sm.red[64][s] = 2.0f * r * inv_n;
+    sm.red[65][s] = r * r;
+  }
+  __syncthreads();
+  const float dout = sm.red[64][s];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    sm.red[c0 + k][s] = dout * v[k];
+    const float sg = sg2[k];
+    v[k] = dout * sm.w3[c0 + k] * (sg * (1.0f + z2[k] * (1.0f - sg)));
+  }
+#pragma unroll
+  for (int k = 0; k < 16; k += 8) st_bf16x8(sm.dz2 + core_offset(s, c0 + k, 8), v + k);
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.ag, c0 + k, s, v[k], v[k + 1]);  // dZ2^T
+  // backpropagation through layer 2
+  tc_issue(sm, tmem, sm.dz2, 1024, sm.w2t, 1024, 4, kIdescN64);
+  if (!tc_await(sm, phase)) return false;
+  tmem_ld16(t_row + uint32_t(c0), v);
+#pragma unroll
+  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.ag, 64 + c0 + k, s, v[k] * d1[k], v[k + 1] * d1[k + 1]);  // dZ1^T
+  // weight and bias gradients of both layers: G = ag bg^T over the tile's samples
+  tc_issue(sm, tmem, sm.ag, 2048, sm.bg, 2048, 8, kIdescN96);
+  // meanwhile w3, b3 and the squared residuals: sums over the tile in sample order (warps 1 to 3)
+  float acc = 0.0f;
+  const int row = tid - 32;
+  if (row >= 0 && row < 66) {
+#pragma unroll 16
+    for (int t = 0; t < kTile; ++t) acc += sm.red[row][t];
+  }
+  if (!tc_await(sm, phase)) return false;
+  if (row >= 0 && row < 64)
+    g[oW3 + row] = acc;
+  else if (row == 64)
+    g[oB3] = acc;
+  else if (row == 65)
+    *sq = acc;
+  // row s of G, columns 24 cg ..: dW2 row s and db2 (s < 64), or dW1 row s - 64 and db1
+  float w[24];
+  tmem_ld16(t_row + uint32_t(cg * 24), w);
+  tmem_ld8(t_row + uint32_t(cg * 24 + 16), w + 16);
+#pragma unroll
+  for (int k = 0; k < 24; ++k) {
+    const int col = cg * 24 + k;
+    if (s < 64) {
+      if (col < 64) g[oW2 + s * 64 + col] = w[k];
+      if (col == 80) g[oB2 + s] = w[k];
+    } else {
+      if (col >= 64 && col < 64 + kIn) g[oW1 + (s - 64) * kIn + (col - 64)] = w[k];
+      if (col == 80) g[oB1 + s - 64] = w[k];
+    }
+  }
+  return true;
+}
+
+__device__ __forceinline__ TrainSmem& train_smem(uint8_t* raw) {
+  // the operands at a 1024-byte boundary (the launch reserves the slack)
+  return *reinterpret_cast<TrainSmem*>(raw + ((1024u - (smem_addr(raw) & 1023u)) & 1023u));
+}
+
+// A wait that ran out: NaN partials (and so a NaN loss), after a bounded time for a product in flight.
+__device__ void train_failed(TrainSmem& sm, uint32_t phase, float* __restrict__ g, float* __restrict__ sq) {
+  const float nan = __int_as_float(0x7fc00000);
+  for (int k = threadIdx.x; k < kMlpParams; k += kTrainThreads) g[k] = nan;
+  if (threadIdx.x == 0) *sq = nan;
+  mbar_wait(&sm.mbar, phase ^ 1u);
+}
+
+// One forward and backward pass over a batch: partial gradients part[CTA], squared residuals sq[CTA].
+__global__ void __launch_bounds__(kTrainThreads, 1)
+    mlp_train_tc_kernel(const float* __restrict__ p, const float* __restrict__ x, int x_stride,
+                        const float* __restrict__ y, int y_stride, uint32_t n, float inv_n, float* __restrict__ part,
+                        float* __restrict__ sq) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  TrainSmem& sm = train_smem(smem_raw);
+  const uint32_t tmem = train_setup(sm);
+  uint32_t phase = 0;
+  train_weights(sm, p);
+  const TrainInput in = train_input(x, x_stride, y, y_stride, n);
+  float* g = part + size_t(blockIdx.x) * kMlpParams;
+  if (!train_tile(sm, tmem, phase, in, n, inv_n, g, sq + blockIdx.x)) train_failed(sm, phase, g, sq + blockIdx.x);
+  train_teardown(tmem);
+}
+
+// One Adam step of a parameter (Kingma & Ba 2015); c1, c2: the bias corrections 1 - beta^t.
+__device__ __forceinline__ void adam(float gk, float& p, float& m, float& v, float lr, float beta1, float beta2, float eps,
+                                     float c1, float c2) {
+  const float mk = beta1 * m + (1.0f - beta1) * gk;
+  const float vk = beta2 * v + (1.0f - beta2) * gk * gk;
+  m = mk;
+  v = vk;
+  p -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
 }
 
 // Sum of the CTAs' partial gradients (in CTA order), written to grad, then (when m is not
@@ -311,13 +441,107 @@ __global__ void __launch_bounds__(256) mlp_reduce_adam_kernel(const float* __res
   for (uint32_t c = 0; c < n_cta; ++c) gk += part[size_t(c) * kMlpParams + k];
   if (grad) grad[k] = gk;
   if (!m) return;
-  const float mk = beta1 * m[k] + (1.0f - beta1) * gk;
-  const float vk = beta2 * v[k] + (1.0f - beta2) * gk * gk;
-  m[k] = mk;
-  v[k] = vk;
-  p[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+  adam(gk, p[k], m[k], v[k], lr, beta1, beta2, eps, c1, c2);
 }
 
+// ---- many training steps in one launch
+// The CTAs of a batch run together (a cooperative launch) and meet twice a step: after writing their
+// partial gradients, and after each has summed its slice of the parameters over the CTAs (in CTA
+// order, as mlp_reduce_adam_kernel does) and taken their Adam step. The moments stay in registers for
+// the launch, the next batch's inputs are loaded before the first meeting. The bias corrections 1 -
+// beta^t come with the launch (kTrainSteps of them), computed on the host.
+constexpr int kTrainSteps = 256;
+constexpr int kSliceMax = (kMlpParams + kTrainThreads - 1) / kTrainThreads;  // parameters a thread, one CTA
+
+struct TrainSteps {
+  const float* records;  // [batches][batch][TKF_MLP_RECORD]
+  uint32_t batch, batches, first, count;  // the launch's steps: first .. first + count - 1 (over all epochs)
+  float *p, *m, *v, *part, *sq, *epoch_loss;
+  uint32_t* meet;  // arrivals of the grid barrier, zeroed before the launch
+  float lr, beta1, beta2, eps;
+  float2 c[kTrainSteps];
+};
+
+// Every CTA of the launch arrives, then waits (bounded) for the others; false if the wait ran out.
+__device__ bool grid_meet(TrainSmem& sm, uint32_t* meet, uint32_t target) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(meet, 1u);
+    uint32_t seen = 0, it = 0;
+    for (; it < (1u << 22); ++it) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(meet) : "memory");
+      if (int32_t(seen - target) >= 0) break;
+      if (it > 4096) __nanosleep(100);
+    }
+    sm.flag = it < (1u << 22);
+    __threadfence();
+  }
+  __syncthreads();
+  return sm.flag != 0;
+}
+
+__global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const __grid_constant__ TrainSteps a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  TrainSmem& sm = train_smem(smem_raw);
+  const uint32_t tmem = train_setup(sm);
+  const uint32_t per = (kMlpParams + gridDim.x - 1) / gridDim.x, k0 = blockIdx.x * per;
+  const uint32_t k1 = min(k0 + per, uint32_t(kMlpParams));
+  float pk[kSliceMax], mk[kSliceMax], vk[kSliceMax];
+#pragma unroll
+  for (int q = 0; q < kSliceMax; ++q) {
+    const uint32_t k = k0 + threadIdx.x + q * kTrainThreads;
+    pk[q] = k < k1 ? a.p[k] : 0.0f;
+    mk[q] = k < k1 ? a.m[k] : 0.0f;
+    vk[q] = k < k1 ? a.v[k] : 0.0f;
+  }
+  const float inv_n = 1.0f / float(a.batch), inv_batches = 1.0f / float(a.batches);
+  float* g = a.part + size_t(blockIdx.x) * kMlpParams;
+  uint32_t phase = 0, met = 0;
+  bool ok = true, together = true;
+  const auto input = [&](uint32_t step) {
+    const float* rec = a.records + size_t(step % a.batches) * a.batch * kMlpRecord;
+    return train_input(rec, kMlpRecord, rec + 12, kMlpRecord, a.batch);
+  };
+  TrainInput in = input(a.first);
+  for (uint32_t i = 0; i < a.count && together; ++i) {
+    train_weights(sm, a.p);
+    if (ok) ok = train_tile(sm, tmem, phase, in, a.batch, inv_n, g, a.sq + blockIdx.x);
+    if (!ok) train_failed(sm, phase, g, a.sq + blockIdx.x);
+    if (i + 1 < a.count) in = input(a.first + i + 1);
+    together = grid_meet(sm, a.meet, (met += gridDim.x));
+    if (!together) break;
+    if (blockIdx.x == 0 && threadIdx.x == kTrainThreads - 1) {
+      float l = 0.0f;
+      for (uint32_t c = 0; c < gridDim.x; ++c) l += __ldcg(a.sq + c);
+      l *= inv_n;
+      a.epoch_loss[(a.first + i) / a.batches] += l * inv_batches;
+    }
+    const float2 c = a.c[i];
+#pragma unroll
+    for (int q = 0; q < kSliceMax; ++q) {
+      const uint32_t k = k0 + threadIdx.x + q * kTrainThreads;
+      if (k < k1) {
+        float gk = 0.0f;
+#pragma unroll 8
+        for (uint32_t cta = 0; cta < gridDim.x; ++cta) gk += __ldcg(a.part + size_t(cta) * kMlpParams + k);
+        adam(gk, pk[q], mk[q], vk[q], a.lr, a.beta1, a.beta2, a.eps, c.x, c.y);
+        a.p[k] = pk[q];
+      }
+    }
+    together = grid_meet(sm, a.meet, (met += gridDim.x));
+  }
+#pragma unroll
+  for (int q = 0; q < kSliceMax; ++q) {
+    const uint32_t k = k0 + threadIdx.x + q * kTrainThreads;
+    if (k < k1) {
+      a.m[k] = mk[q];
+      a.v[k] = vk[q];
+      if (!together) a.p[k] = __int_as_float(0x7fc00000);
+    }
+  }
+  train_teardown(tmem);
+}
 
 // ---- initialisation: W ~ U(-1/sqrt(fan_in), 1/sqrt(fan_in)) from SplitMix64 of (seed, index), b = 0
 __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
@@ -451,30 +675,52 @@ cudaError_t mlp_round_bf16(const float* in, float* out, uint32_t* bad, cudaStrea
 
 size_t mlp_train_scratch_bytes(uint32_t batch) {
   const size_t n_cta = (size_t(batch) + kTile - 1) / kTile;
-  return sizeof(float) * (n_cta * (kMlpParams + 1) + kMlpParams) + 256;
+  return sizeof(float) * (n_cta * (kMlpParams + 1) + kMlpParams + 1) + 256;
 }
 
 namespace {
-// Partial gradients [n_cta][params], per-CTA squared residuals [n_cta], the summed gradient.
+// Partial gradients [n_cta][params], per-CTA squared residuals [n_cta], the summed gradient, the
+// arrivals of the steps kernel's grid barrier.
 struct TrainScratch {
   float* part;
   float* sq;
   float* grad;
+  uint32_t* meet;
 };
 TrainScratch carve_train(void* base, uint32_t batch) {
   const size_t n_cta = (size_t(batch) + kTile - 1) / kTile;
   float* f = static_cast<float*>(base);
-  return TrainScratch{f, f + n_cta * kMlpParams, f + n_cta * (kMlpParams + 1)};
+  float* grad = f + n_cta * (kMlpParams + 1);
+  return TrainScratch{f, f + n_cta * kMlpParams, grad, reinterpret_cast<uint32_t*>(grad + kMlpParams)};
+}
+
+constexpr size_t kTrainSmemBytes = sizeof(TrainSmem) + 1024;  // + alignment slack
+static_assert(kTrainSmemBytes <= 227 * 1024, "shared memory");
+
+// Whether a batch's CTAs can run at the same time on this device (one an SM), as the steps kernel
+// needs; the largest batch has 64. A device partition with fewer SMs trains step by step.
+bool train_together(unsigned n_cta) {
+  int dev = 0, sms = 0, coop = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+      cudaFuncSetAttribute(mlp_train_steps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTrainSmemBytes)) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_steps_kernel, kTrainThreads, kTrainSmemBytes) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return coop && n_cta <= unsigned(sms) * unsigned(per_sm);
 }
 
 cudaError_t train_tile_launch(const float* params, const float* x, int x_stride, const float* y, int y_stride,
                               uint32_t n, const TrainScratch& sc, cudaStream_t stream) {
-  static_assert(sizeof(TrainSmem) + 1024 <= 227 * 1024, "shared memory");
-  const size_t smem = sizeof(TrainSmem) + 1024;  // + alignment slack
-  cudaError_t e = cudaFuncSetAttribute(mlp_train_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  cudaError_t e = cudaFuncSetAttribute(mlp_train_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(kTrainSmemBytes));
   if (e != cudaSuccess) return e;
   const unsigned n_cta = (n + kTile - 1) / kTile;
-  mlp_train_tc_kernel<<<n_cta, kTile, smem, stream>>>(params, x, x_stride, y, y_stride, n, 1.0f / float(n), sc.part,
+  mlp_train_tc_kernel<<<n_cta, kTrainThreads, kTrainSmemBytes, stream>>>(params, x, x_stride, y, y_stride, n, 1.0f / float(n), sc.part,
                                                       sc.sq);
   return cudaGetLastError();
 }
@@ -500,16 +746,54 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
   const unsigned n_cta = (batch + kTile - 1) / kTile;
   cudaError_t e = cudaMemsetAsync(epoch_loss, 0, sizeof(float) * epochs, stream);
   if (e != cudaSuccess) return e;
+  const uint64_t steps = uint64_t(epochs) * nb;
+  const auto corrections = [&](uint32_t t) {
+    return make_float2(1.0f - powf(beta1, float(t)), 1.0f - powf(beta2, float(t)));
+  };
+  if (steps > 0 && steps < (uint64_t(1) << 32) && train_together(n_cta)) {  // many steps a launch
+    TrainSteps a{};
+    a.records = records;
+    a.batch = batch;
+    a.batches = nb;
+    a.p = params;
+    a.m = moments;
+    a.v = moments + kMlpParams;
+    a.part = sc.part;
+    a.sq = sc.sq;
+    a.epoch_loss = epoch_loss;
+    a.meet = sc.meet;
+    a.lr = lr;
+    a.beta1 = beta1;
+    a.beta2 = beta2;
+    a.eps = eps;
+    for (uint64_t done = 0; done < steps; done += a.count) {
+      a.first = uint32_t(done);
+      a.count = uint32_t(steps - done < uint64_t(kTrainSteps) ? steps - done : uint64_t(kTrainSteps));
+      for (uint32_t i = 0; i < a.count; ++i) a.c[i] = corrections(++(*adam_t));
+      if ((e = cudaMemsetAsync(sc.meet, 0, sizeof(uint32_t), stream)) != cudaSuccess) return e;
+      cudaLaunchAttribute attr{};
+      attr.id = cudaLaunchAttributeCooperative;
+      attr.val.cooperative = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(n_cta);
+      cfg.blockDim = dim3(kTrainThreads);
+      cfg.dynamicSmemBytes = kTrainSmemBytes;
+      cfg.stream = stream;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if ((e = cudaLaunchKernelEx(&cfg, mlp_train_steps_kernel, a)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   for (uint32_t ep = 0; ep < epochs; ++ep) {
     for (uint32_t b = 0; b < nb; ++b) {
       const float* rec = records + size_t(b) * batch * kMlpRecord;
       e = train_tile_launch(params, rec, kMlpRecord, rec + 12, kMlpRecord, batch, sc, stream);
       if (e != cudaSuccess) return e;
-      const uint32_t t = ++(*adam_t);
-      const float c1 = 1.0f - powf(beta1, float(t)), c2 = 1.0f - powf(beta2, float(t));
+      const float2 c = corrections(++(*adam_t));
       mlp_reduce_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(
           sc.part, sc.sq, n_cta, 1.0f / float(batch), sc.grad, params, moments, moments + kMlpParams, lr, beta1, beta2,
-          eps, c1, c2, nullptr, epoch_loss + ep, 1.0f / float(nb));
+          eps, c.x, c.y, nullptr, epoch_loss + ep, 1.0f / float(nb));
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
