@@ -20,6 +20,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "tkf_fit_impl.cuh"
 
 namespace tkf {
@@ -93,11 +95,13 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const float* __restric
 // BF16 operands are rounded to nearest even from the FP32 values; the products are exact and
 // summed in FP32.
 //
-// A step's work is tiny (8 tiles at batch 1024) and serial: it is bound by latencies, not by the
-// tensor cores. With one thread a sample and two launches a step it took 42 us (a 32-way bank
-// conflict in the tile's sums alone 4 us); four threads a sample, padded sums that overlap the last
-// product, and many steps a launch (mlp_train_steps_kernel) bring it to 17 us
-// (two epochs of 380,000 records: 31.7 -> 12.9 ms, the same bits).
+// A step's work is tiny (8 tiles at batch 1024) and serial: it is bound by latencies and by the issue
+// slots of the SMs that hold its tiles, not by the tensor cores. With one thread a sample and two
+// launches a step it took 42 us; four threads a sample, padded sums that overlap the last product, and
+// many steps a launch brought it to 17 us; the CTAs of a batch as one cluster, partial gradients in the
+// product's order, BF16 pairs rounded and stored by the word, and no block-wide vote after each product
+// to 12 us (two epochs of 380,000 records: 31.7 -> 12.9 -> 8.8 ms, the same bits). What is left: the
+// SiLU's exponentials and divisions 6 of 22 kcycles, four products' round trips 3.4, two barriers 2.8.
 constexpr int kTile = 128;
 constexpr int kTrainThreads = 512;
 constexpr uint32_t kIdescN64 = umma_idesc_bf16(128, 64);
@@ -113,8 +117,10 @@ struct __align__(1024) TrainSmem {
   uint8_t w2t[64 * 64 * 2];   // W2^T (N = i, K = j)
   uint8_t xa[128 * 16 * 2];
   uint8_t w1[64 * 16 * 2];    // W1 (N = j, K = inputs, 12..15 zero)
+  float xs[kTile * kMlpRecord];  // a tile's records (the steps kernel)
   float red[66][kTile + 1];   // per-sample a2[j], then dout a2[j] (j < 64), dout, squared residual; padded
-  float b1[64], b2[64], w3[64], b3;
+  alignas(16) float b1[64];
+  float b2[64], w3[64], b3;
   uint64_t mbar;
   uint32_t tmem_base, flag;
 };
@@ -178,32 +184,38 @@ __device__ void tc_issue(TrainSmem& sm, uint32_t tmem, const uint8_t* a, uint32_
     tc_commit(&sm.mbar);
   }
 }
-// Waits for it (every thread, bounded). Returns false, in every thread, if a wait ran out.
-__device__ bool tc_await(TrainSmem& sm, uint32_t& phase) {
+// Waits for it (every thread, bounded); false if this thread's wait ran out. The tile goes on regardless
+// (its values are then discarded), so that every thread passes the same barriers.
+__device__ __forceinline__ bool tc_await(TrainSmem& sm, uint32_t& phase) {
   const bool done = mbar_poll(&sm.mbar, phase);
   phase ^= 1u;
   __syncwarp();
   tc_fence_after();
-  return __syncthreads_or(!done) == 0;
+  return done;
 }
 
-// A value of row `j` (even) and of row j + 1 at K = this thread's sample, into an operand with 16 K
-// groups: lane pairs (consecutive samples) exchange one value each, so that a lane stores one 32-bit
+// Two FP32 values rounded to BF16 (nearest even), lo in the low half.
+__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
+}
+
+// A value of row `r` and of row r + 1 at K index `k`, with k + 1 at the next lane for even lanes, into an
+// operand with `kgroups` K groups: lane pairs exchange one value each, so that a lane stores one 32-bit
 // word of one row.
-__device__ __forceinline__ void st_bf16_pair(uint8_t* base, int j, int s, float v0, float v1) {
-  const uint32_t lane = threadIdx.x & 31u, odd = lane & 1u;
-  const uint32_t b0 = bf16_rne(v0), b1 = bf16_rne(v1);
-  const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? b0 : b1, 1);
-  const uint32_t word = odd ? (got | (b1 << 16)) : (b0 | (got << 16));
-  *reinterpret_cast<uint32_t*>(base + core_offset(j + int(odd), s & ~1, 16)) = word;
+__device__ __forceinline__ void st_bf16_pair(uint8_t* base, int r, int k, int kgroups, float v0, float v1) {
+  const uint32_t odd = threadIdx.x & 1u, b = bf16x2(v0, v1);
+  const uint32_t got = __shfl_xor_sync(0xffffffffu, b, 1);
+  // even: own v0, the neighbour's v0; odd: the neighbour's v1, own v1
+  const uint32_t word = odd ? __byte_perm(got, b, 0x7632) : __byte_perm(b, got, 0x5410);
+  *reinterpret_cast<uint32_t*>(base + core_offset(r + int(odd), k & ~1, kgroups)) = word;
 }
 
 // 8 consecutive K values of one row of an operand (one 16-byte store)
 __device__ __forceinline__ void st_bf16x8(uint8_t* at, const float* v) {
-  uint32_t w[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) w[q] = bf16_rne(v[2 * q]) | (bf16_rne(v[2 * q + 1]) << 16);
-  *reinterpret_cast<uint4*>(at) = make_uint4(w[0], w[1], w[2], w[3]);
+  *reinterpret_cast<uint4*>(at) =
+      make_uint4(bf16x2(v[0], v[1]), bf16x2(v[2], v[3]), bf16x2(v[4], v[5]), bf16x2(v[6], v[7]));
 }
 
 // One CTA's set-up: mbarrier, 128 accumulator columns (each stage writes from column 0), the operands'
@@ -235,33 +247,57 @@ __device__ void train_teardown(uint32_t tmem) {
   }
 }
 
-// Parameters as BF16 operands (both orientations of W2), biases and w3 in FP32. The loads skip L1: the
-// parameters change between the steps of one launch.
-__device__ void train_weights(TrainSmem& sm, const float* __restrict__ p) {
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int q = 0; q < 64 * 16 / kTrainThreads; ++q) {
-    const int e = tid + q * kTrainThreads, j = e >> 4, i = e & 15;
-    st_bf16(sm.w1, core_offset(j, i, 2), i < kIn ? __ldcg(p + oW1 + j * kIn + i) : 0.0f);
-  }
-  float w[64 * 64 / kTrainThreads];
-#pragma unroll
-  for (int q = 0; q < 64 * 64 / kTrainThreads; ++q) w[q] = __ldcg(p + oW2 + tid + q * kTrainThreads);
-#pragma unroll
-  for (int q = 0; q < 64 * 64 / kTrainThreads; ++q) {
-    const int e = tid + q * kTrainThreads, j = e >> 6, i = e & 63;
-    st_bf16(sm.w2, core_offset(j, i, 8), w[q]);
-    st_bf16(sm.w2t, core_offset(i, j, 8), w[q]);
-  }
-  if (tid < 64)
-    sm.b1[tid] = __ldcg(p + oB1 + tid);
-  else if (tid < 128)
-    sm.b2[tid - 64] = __ldcg(p + oB2 + tid - 64);
-  else if (tid < 192)
-    sm.w3[tid - 128] = __ldcg(p + oW3 + tid - 128);
-  else if (tid == 192)
-    sm.b3 = __ldcg(p + oB3);
+// Partial gradients, and the parameters while many steps train them, are kept in the order in which the
+// gradient product leaves them (lane = row of G): W2 by columns (i 64 + j), then W1 by columns, b2, b1,
+// w3, b3. A warp then stores and loads whole lines; row by row the stores of one step took 3 us.
+constexpr int gW1 = 4096, gB2 = 4864, gB1 = 4928;
+__host__ __device__ __forceinline__ int g_index(int k) {  // place of parameter k
+  if (k < oB1) return gW1 + (k % kIn) * 64 + k / kIn;
+  if (k < oW2) return gB1 + (k - oB1);
+  if (k < oB2) return ((k - oW2) & 63) * 64 + ((k - oW2) >> 6);
+  if (k < oW3) return gB2 + (k - oB2);
+  return k;
 }
+__device__ __forceinline__ int g_param(int e) {  // parameter at place e
+  if (e < gW1) return oW2 + (e & 63) * 64 + (e >> 6);
+  if (e < gB2) return oW1 + (e & 63) * kIn + ((e - gW1) >> 6);
+  if (e < gB1) return oB2 + (e - gB2);
+  if (e < oW3) return oB1 + (e - gB1);
+  return e;
+}
+
+// Parameters (in that order, kG, or as the caller keeps them) as BF16 operands (both orientations of
+// W2), biases and w3 in FP32. The loads skip L1 (the parameters change between the steps of one launch)
+// and are all issued before the first store.
+template <bool kG>
+__device__ void train_weights(TrainSmem& sm, const float* __restrict__ p) {
+  const int tid = threadIdx.x, j = tid & 63, ig = tid >> 6;  // row j, columns 8 ig .. (W2) and 2 ig .. (W1)
+  const auto at = [&](int k) { return __ldcg(p + (kG ? g_index(k) : k)); };
+  float w2[8], w1[2], b = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) w2[q] = at(oW2 + j * 64 + ig * 8 + q);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) w1[q] = ig * 2 + q < kIn ? at(oW1 + j * kIn + ig * 2 + q) : 0.0f;
+  if (tid < 64)
+    b = at(oB1 + tid);
+  else if (tid < 128)
+    b = at(oB2 + tid - 64);
+  else if (tid <= 192)
+    b = at(oW3 + tid - 128);  // w3, then b3
+  st_bf16x8(sm.w2 + core_offset(j, ig * 8, 8), w2);
+#pragma unroll
+  for (int q = 0; q < 8; q += 2) st_bf16_pair(sm.w2t, ig * 8 + q, j, 8, w2[q], w2[q + 1]);
+  *reinterpret_cast<uint32_t*>(sm.w1 + core_offset(j, ig * 2, 2)) = bf16x2(w1[0], w1[1]);
+  if (tid < 64)
+    sm.b1[tid] = b;
+  else if (tid < 128)
+    sm.b2[tid - 64] = b;
+  else if (tid < 192)
+    sm.w3[tid - 128] = b;
+  else if (tid == 192)
+    sm.b3 = b;
+}
+static_assert(kTrainThreads == 512, "eight threads a row of W2");
 
 // This thread's quarter of its sample's inputs (4 of 16, the last four zero) and the label.
 struct TrainInput {
@@ -279,23 +315,49 @@ __device__ __forceinline__ TrainInput train_input(const float* __restrict__ x, i
   return in;
 }
 
+// The same from records (inputs, label), whose tile is contiguous: whole lines into registers (ahead of
+// time), then by way of shared memory; thread by thread the strided loads of a step took 1.5 us.
+constexpr int kTileLoads = (kTile * kMlpRecord + kTrainThreads - 1) / kTrainThreads;
+__device__ __forceinline__ void tile_records(const float* __restrict__ rec, uint32_t n, float v[kTileLoads]) {
+  const uint32_t from = blockIdx.x * kTile * kMlpRecord;
+#pragma unroll
+  for (int q = 0; q < kTileLoads; ++q) {
+    const uint32_t e = threadIdx.x + q * kTrainThreads;
+    v[q] = e < kTile * kMlpRecord && from + e < n * kMlpRecord ? rec[from + e] : 0.0f;
+  }
+}
+__device__ __forceinline__ TrainInput tile_input(TrainSmem& sm, const float v[kTileLoads]) {
+  const uint32_t s = threadIdx.x & (kTile - 1), cg = threadIdx.x >> 7;
+#pragma unroll
+  for (int q = 0; q < kTileLoads; ++q) {
+    const uint32_t e = threadIdx.x + q * kTrainThreads;
+    if (e < kTile * kMlpRecord) sm.xs[e] = v[q];
+  }
+  __syncthreads();
+  TrainInput in;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) in.x[i] = cg < kIn / 4 ? sm.xs[s * kMlpRecord + cg * 4 + i] : 0.0f;
+  in.y = sm.xs[s * kMlpRecord + 12];
+  return in;
+}
+
 // Forward and backward pass of one tile; the CTA's partial gradient (TKF_MLP_PARAMS floats) and
 // its sum of squared residuals go to g and *sq. `inv_n`: 1 / batch size (dL/dout = 2 r / n). Returns
-// false (nothing written) if a wait for the tensor cores ran out.
+// false (nothing written) if any thread's wait for the tensor cores ran out.
 __device__ bool train_tile(TrainSmem& sm, uint32_t tmem, uint32_t& phase, const TrainInput& in, uint32_t n, float inv_n,
                            float* __restrict__ g, float* __restrict__ sq) {
   const int tid = threadIdx.x, s = tid & (kTile - 1), cg = tid >> 7, c0 = cg * 16;
   const bool live = blockIdx.x * kTile + s < n;
   const uint32_t t_row = tmem + (uint32_t(s & ~31) << 16);  // this warp's 32 lanes
   for (int i = 0; i < 4; i += 2) {
-    st_bf16(sm.xa, core_offset(s, cg * 4 + i, 2), in.x[i]);
-    st_bf16(sm.xa, core_offset(s, cg * 4 + i + 1, 2), in.x[i + 1]);
-    st_bf16_pair(sm.bg, 64 + cg * 4 + i, s, in.x[i], in.x[i + 1]);  // X^T
+    *reinterpret_cast<uint32_t*>(sm.xa + core_offset(s, cg * 4 + i, 2)) = bf16x2(in.x[i], in.x[i + 1]);
+    st_bf16_pair(sm.bg, 64 + cg * 4 + i, s, 16, in.x[i], in.x[i + 1]);  // X^T
   }
+  bool ok = true;
   float v[16], d1[16], z2[16], sg2[16];  // d1: SiLU'(Z1 + b1)
   // layer 1
   tc_issue(sm, tmem, sm.xa, 256, sm.w1, 256, 1, kIdescN64);
-  if (!tc_await(sm, phase)) return false;
+  ok = tc_await(sm, phase) && ok;
   tmem_ld16(t_row + uint32_t(c0), v);
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
@@ -306,10 +368,10 @@ __device__ bool train_tile(TrainSmem& sm, uint32_t tmem, uint32_t& phase, const 
 #pragma unroll
   for (int k = 0; k < 16; k += 8) st_bf16x8(sm.a1 + core_offset(s, c0 + k, 8), v + k);
 #pragma unroll
-  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.bg, c0 + k, s, v[k], v[k + 1]);  // A1^T
+  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.bg, c0 + k, s, 16, v[k], v[k + 1]);  // A1^T
   // layer 2
   tc_issue(sm, tmem, sm.a1, 1024, sm.w2, 1024, 4, kIdescN64);
-  if (!tc_await(sm, phase)) return false;
+  ok = tc_await(sm, phase) && ok;
   tmem_ld16(t_row + uint32_t(c0), v);
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
@@ -338,13 +400,13 @@ __device__ bool train_tile(TrainSmem& sm, uint32_t tmem, uint32_t& phase, const 
 #pragma unroll
   for (int k = 0; k < 16; k += 8) st_bf16x8(sm.dz2 + core_offset(s, c0 + k, 8), v + k);
 #pragma unroll
-  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.ag, c0 + k, s, v[k], v[k + 1]);  // dZ2^T
+  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.ag, c0 + k, s, 16, v[k], v[k + 1]);  // dZ2^T
   // backpropagation through layer 2
   tc_issue(sm, tmem, sm.dz2, 1024, sm.w2t, 1024, 4, kIdescN64);
-  if (!tc_await(sm, phase)) return false;
+  ok = tc_await(sm, phase) && ok;
   tmem_ld16(t_row + uint32_t(c0), v);
 #pragma unroll
-  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.ag, 64 + c0 + k, s, v[k] * d1[k], v[k + 1] * d1[k + 1]);  // dZ1^T
+  for (int k = 0; k < 16; k += 2) st_bf16_pair(sm.ag, 64 + c0 + k, s, 16, v[k] * d1[k], v[k + 1] * d1[k + 1]);  // dZ1^T
   // weight and bias gradients of both layers: G = ag bg^T over the tile's samples
   tc_issue(sm, tmem, sm.ag, 2048, sm.bg, 2048, 8, kIdescN96);
   // meanwhile w3, b3 and the squared residuals: sums over the tile in sample order (warps 1 to 3)
@@ -354,7 +416,9 @@ __device__ bool train_tile(TrainSmem& sm, uint32_t tmem, uint32_t& phase, const 
 #pragma unroll 16
     for (int t = 0; t < kTile; ++t) acc += sm.red[row][t];
   }
-  if (!tc_await(sm, phase)) return false;
+  ok = tc_await(sm, phase) && ok;
+  ok = __syncthreads_or(!ok) == 0;
+  if (!ok) return false;
   if (row >= 0 && row < 64)
     g[oW3 + row] = acc;
   else if (row == 64)
@@ -369,14 +433,14 @@ __device__ bool train_tile(TrainSmem& sm, uint32_t tmem, uint32_t& phase, const 
   for (int k = 0; k < 24; ++k) {
     const int col = cg * 24 + k;
     if (s < 64) {
-      if (col < 64) g[oW2 + s * 64 + col] = w[k];
-      if (col == 80) g[oB2 + s] = w[k];
+      if (col < 64) g[col * 64 + s] = w[k];
+      if (col == 80) g[gB2 + s] = w[k];
     } else {
-      if (col >= 64 && col < 64 + kIn) g[oW1 + (s - 64) * kIn + (col - 64)] = w[k];
-      if (col == 80) g[oB1 + s - 64] = w[k];
+      if (col >= 64 && col < 64 + kIn) g[gW1 + (col - 64) * 64 + s - 64] = w[k];
+      if (col == 80) g[gB1 + s - 64] = w[k];
     }
   }
-  return true;
+  return ok;
 }
 
 __device__ __forceinline__ TrainSmem& train_smem(uint8_t* raw) {
@@ -401,7 +465,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   TrainSmem& sm = train_smem(smem_raw);
   const uint32_t tmem = train_setup(sm);
   uint32_t phase = 0;
-  train_weights(sm, p);
+  train_weights<false>(sm, p);
   const TrainInput in = train_input(x, x_stride, y, y_stride, n);
   float* g = part + size_t(blockIdx.x) * kMlpParams;
   if (!train_tile(sm, tmem, phase, in, n, inv_n, g, sq + blockIdx.x)) train_failed(sm, phase, g, sq + blockIdx.x);
@@ -438,7 +502,7 @@ __global__ void __launch_bounds__(256) mlp_reduce_adam_kernel(const float* __res
   }
   if (k >= kMlpParams) return;
   float gk = 0.0f;
-  for (uint32_t c = 0; c < n_cta; ++c) gk += part[size_t(c) * kMlpParams + k];
+  for (uint32_t c = 0; c < n_cta; ++c) gk += part[size_t(c) * kMlpParams + g_index(k)];
   if (grad) grad[k] = gk;
   if (!m) return;
   adam(gk, p[k], m[k], v[k], lr, beta1, beta2, eps, c1, c2);
@@ -457,59 +521,74 @@ struct TrainSteps {
   const float* records;  // [batches][batch][TKF_MLP_RECORD]
   uint32_t batch, batches, first, count;  // the launch's steps: first .. first + count - 1 (over all epochs)
   float *p, *m, *v, *part, *sq, *epoch_loss;
+  float* q;        // the parameters in the gradient's order, for the launch
   uint32_t* meet;  // arrivals of the grid barrier, zeroed before the launch
   float lr, beta1, beta2, eps;
   float2 c[kTrainSteps];
 };
 
-// Every CTA of the launch arrives, then waits (bounded) for the others; false if the wait ran out.
-__device__ bool grid_meet(TrainSmem& sm, uint32_t* meet, uint32_t target) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(meet, 1u);
-    uint32_t seen = 0, it = 0;
-    for (; it < (1u << 22); ++it) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(meet) : "memory");
-      if (int32_t(seen - target) >= 0) break;
-      if (it > 4096) __nanosleep(100);
+// Every CTA of the launch arrives, then waits for the others: by the hardware barrier where the CTAs are
+// one cluster, else by a counter (bounded: false if the wait ran out).
+template <bool kCluster>
+__device__ bool train_meet(TrainSmem& sm, uint32_t* meet, uint32_t target) {
+  if constexpr (kCluster) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  } else {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      atomicAdd(meet, 1u);
+      uint32_t seen = 0, it = 0;
+      for (; it < (1u << 22); ++it) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(meet) : "memory");
+        if (int32_t(seen - target) >= 0) break;
+        if (it > 4096) __nanosleep(100);
+      }
+      sm.flag = it < (1u << 22);
+      __threadfence();
     }
-    sm.flag = it < (1u << 22);
-    __threadfence();
+    __syncthreads();
+    return sm.flag != 0;
   }
-  __syncthreads();
-  return sm.flag != 0;
 }
 
+template <bool kCluster>
 __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const __grid_constant__ TrainSteps a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   TrainSmem& sm = train_smem(smem_raw);
   const uint32_t tmem = train_setup(sm);
-  const uint32_t per = (kMlpParams + gridDim.x - 1) / gridDim.x, k0 = blockIdx.x * per;
-  const uint32_t k1 = min(k0 + per, uint32_t(kMlpParams));
+  // this CTA's slice of the parameters, in the gradient's order
+  const uint32_t per = (kMlpParams + gridDim.x - 1) / gridDim.x, e0 = blockIdx.x * per;
+  const uint32_t e1 = min(e0 + per, uint32_t(kMlpParams));
   float pk[kSliceMax], mk[kSliceMax], vk[kSliceMax];
 #pragma unroll
   for (int q = 0; q < kSliceMax; ++q) {
-    const uint32_t k = k0 + threadIdx.x + q * kTrainThreads;
-    pk[q] = k < k1 ? a.p[k] : 0.0f;
-    mk[q] = k < k1 ? a.m[k] : 0.0f;
-    vk[q] = k < k1 ? a.v[k] : 0.0f;
+    const uint32_t e = e0 + threadIdx.x + q * kTrainThreads;
+    const int k = e < e1 ? g_param(int(e)) : 0;
+    pk[q] = a.p[k];
+    mk[q] = a.m[k];
+    vk[q] = a.v[k];
+    if (e < e1) a.q[e] = pk[q];
   }
   const float inv_n = 1.0f / float(a.batch), inv_batches = 1.0f / float(a.batches);
   float* g = a.part + size_t(blockIdx.x) * kMlpParams;
   uint32_t phase = 0, met = 0;
-  bool ok = true, together = true;
-  const auto input = [&](uint32_t step) {
-    const float* rec = a.records + size_t(step % a.batches) * a.batch * kMlpRecord;
-    return train_input(rec, kMlpRecord, rec + 12, kMlpRecord, a.batch);
+  bool ok = true;
+  float rec[kTileLoads];
+  const auto load = [&](uint32_t step) {
+    tile_records(a.records + size_t(step % a.batches) * a.batch * kMlpRecord, a.batch, rec);
   };
-  TrainInput in = input(a.first);
+  load(a.first);
+  bool together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x));  // every slice of q is there
   for (uint32_t i = 0; i < a.count && together; ++i) {
-    train_weights(sm, a.p);
+    train_weights<true>(sm, a.q);
+    const TrainInput in = tile_input(sm, rec);
     if (ok) ok = train_tile(sm, tmem, phase, in, a.batch, inv_n, g, a.sq + blockIdx.x);
     if (!ok) train_failed(sm, phase, g, a.sq + blockIdx.x);
-    if (i + 1 < a.count) in = input(a.first + i + 1);
-    together = grid_meet(sm, a.meet, (met += gridDim.x));
+    if (i + 1 < a.count) load(a.first + i + 1);
+    together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x));
     if (!together) break;
     if (blockIdx.x == 0 && threadIdx.x == kTrainThreads - 1) {
       float l = 0.0f;
@@ -518,26 +597,42 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const
       a.epoch_loss[(a.first + i) / a.batches] += l * inv_batches;
     }
     const float2 c = a.c[i];
+    // every element's sum runs over the CTAs in order; the loads of a thread's elements overlap
+    const auto reduce = [&](auto n_elements) {
+      constexpr int kN = decltype(n_elements)::value;
+      float gk[kN];
 #pragma unroll
-    for (int q = 0; q < kSliceMax; ++q) {
-      const uint32_t k = k0 + threadIdx.x + q * kTrainThreads;
-      if (k < k1) {
-        float gk = 0.0f;
+      for (int q = 0; q < kN; ++q) gk[q] = 0.0f;
+      const float* at = a.part + e0 + threadIdx.x;
 #pragma unroll 8
-        for (uint32_t cta = 0; cta < gridDim.x; ++cta) gk += __ldcg(a.part + size_t(cta) * kMlpParams + k);
-        adam(gk, pk[q], mk[q], vk[q], a.lr, a.beta1, a.beta2, a.eps, c.x, c.y);
-        a.p[k] = pk[q];
+      for (uint32_t cta = 0; cta < gridDim.x; ++cta, at += kMlpParams) {
+#pragma unroll
+        for (int q = 0; q < kN; ++q)
+          if (e0 + threadIdx.x + q * kTrainThreads < e1) gk[q] += __ldcg(at + q * kTrainThreads);
       }
-    }
-    together = grid_meet(sm, a.meet, (met += gridDim.x));
+#pragma unroll
+      for (int q = 0; q < kN; ++q) {
+        const uint32_t e = e0 + threadIdx.x + q * kTrainThreads;
+        if (e < e1) {
+          adam(gk[q], pk[q], mk[q], vk[q], a.lr, a.beta1, a.beta2, a.eps, c.x, c.y);
+          a.q[e] = pk[q];
+        }
+      }
+    };
+    if (per <= 2 * kTrainThreads)
+      reduce(std::integral_constant<int, 2>{});
+    else
+      reduce(std::integral_constant<int, kSliceMax>{});
+    together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x));
   }
 #pragma unroll
   for (int q = 0; q < kSliceMax; ++q) {
-    const uint32_t k = k0 + threadIdx.x + q * kTrainThreads;
-    if (k < k1) {
+    const uint32_t e = e0 + threadIdx.x + q * kTrainThreads;
+    if (e < e1) {
+      const int k = g_param(int(e));
       a.m[k] = mk[q];
       a.v[k] = vk[q];
-      if (!together) a.p[k] = __int_as_float(0x7fc00000);
+      a.p[k] = together ? pk[q] : __int_as_float(0x7fc00000);
     }
   }
   train_teardown(tmem);
@@ -675,23 +770,25 @@ cudaError_t mlp_round_bf16(const float* in, float* out, uint32_t* bad, cudaStrea
 
 size_t mlp_train_scratch_bytes(uint32_t batch) {
   const size_t n_cta = (size_t(batch) + kTile - 1) / kTile;
-  return sizeof(float) * (n_cta * (kMlpParams + 1) + kMlpParams + 1) + 256;
+  return sizeof(float) * (n_cta * (kMlpParams + 1) + 2 * kMlpParams + 1) + 256;
 }
 
 namespace {
-// Partial gradients [n_cta][params], per-CTA squared residuals [n_cta], the summed gradient, the
-// arrivals of the steps kernel's grid barrier.
+// Partial gradients [n_cta][params], per-CTA squared residuals [n_cta], the summed gradient, the steps
+// kernel's parameters and the arrivals of its grid barrier.
 struct TrainScratch {
   float* part;
   float* sq;
   float* grad;
+  float* q;
   uint32_t* meet;
 };
 TrainScratch carve_train(void* base, uint32_t batch) {
   const size_t n_cta = (size_t(batch) + kTile - 1) / kTile;
   float* f = static_cast<float*>(base);
   float* grad = f + n_cta * (kMlpParams + 1);
-  return TrainScratch{f, f + n_cta * kMlpParams, grad, reinterpret_cast<uint32_t*>(grad + kMlpParams)};
+  return TrainScratch{f, f + n_cta * kMlpParams, grad, grad + kMlpParams,
+                      reinterpret_cast<uint32_t*>(grad + 2 * kMlpParams)};
 }
 
 constexpr size_t kTrainSmemBytes = sizeof(TrainSmem) + 1024;  // + alignment slack
@@ -704,10 +801,12 @@ bool train_together(unsigned n_cta) {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaFuncSetAttribute(mlp_train_steps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTrainSmemBytes)) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_steps_kernel, kTrainThreads, kTrainSmemBytes) !=
-          cudaSuccess) {
+      cudaFuncSetAttribute(mlp_train_steps_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(kTrainSmemBytes)) != cudaSuccess ||
+      cudaFuncSetAttribute(mlp_train_steps_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(kTrainSmemBytes)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_steps_kernel<false>, kTrainThreads,
+                                                    kTrainSmemBytes) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -761,7 +860,10 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
     a.part = sc.part;
     a.sq = sc.sq;
     a.epoch_loss = epoch_loss;
+    a.q = sc.q;
     a.meet = sc.meet;
+    // 2, 4 or 8 CTAs (batches of 129 to 1024) as one cluster: its barrier takes a fifth of the counter's time
+    const bool cluster = n_cta == 2 || n_cta == 4 || n_cta == 8;
     a.lr = lr;
     a.beta1 = beta1;
     a.beta2 = beta2;
@@ -772,8 +874,14 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
       for (uint32_t i = 0; i < a.count; ++i) a.c[i] = corrections(++(*adam_t));
       if ((e = cudaMemsetAsync(sc.meet, 0, sizeof(uint32_t), stream)) != cudaSuccess) return e;
       cudaLaunchAttribute attr{};
-      attr.id = cudaLaunchAttributeCooperative;
-      attr.val.cooperative = 1;
+      if (cluster) {
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = n_cta;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      } else {
+        attr.id = cudaLaunchAttributeCooperative;
+        attr.val.cooperative = 1;
+      }
       cudaLaunchConfig_t cfg{};
       cfg.gridDim = dim3(n_cta);
       cfg.blockDim = dim3(kTrainThreads);
@@ -781,7 +889,9 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
       cfg.stream = stream;
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
-      if ((e = cudaLaunchKernelEx(&cfg, mlp_train_steps_kernel, a)) != cudaSuccess) return e;
+      e = cluster ? cudaLaunchKernelEx(&cfg, mlp_train_steps_kernel<true>, a)
+                  : cudaLaunchKernelEx(&cfg, mlp_train_steps_kernel<false>, a);
+      if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
   }
