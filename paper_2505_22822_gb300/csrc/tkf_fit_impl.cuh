@@ -21,39 +21,17 @@
 
 #include <math.h>
 
+#include "tkf_fp64.cuh"
 #include "tkf_internal.cuh"
 
 namespace tkf {
 namespace {
 
 constexpr double kKappa = 2.99792458e-4;  // GeV / (T mm)
-constexpr double kPi = 3.14159265358979323846;
 constexpr double kMe = 0.51099895e-3;  // GeV
 constexpr double kBetheK = 0.307075;   // MeV cm^2 / mol
 
 constexpr uint32_t kFatal = ~(TKF_TRACK_TOO_FEW_HITS | TKF_TRACK_OUT_OF_FIELD | TKF_TRACK_PROPOSAL_FALLBACK);
-
-// Exact FP32 <-> FP64 conversions on the integer pipes. On GB300 the hardware conversion runs
-// on the FP64 pipe (a warp instruction occupies it for 16 SM cycles), and the FP64 pipe bounds
-// the mixed path; these give the IEEE results (round to nearest even) for every normal number
-// and zero with a few integer operations. FP32 denormals become signed zero; out of range
-// FP64 values (beyond the FP32 normals, infinities, NaN) become NaN, and FP32 infinities and
-// NaN become FP64 NaN, so a non-finite value stays non-finite.
-__device__ __forceinline__ double f2d(float x) {
-  const uint32_t u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
-  const bool tiny = a < 0x00800000u, special = a >= 0x7F800000u;
-  const uint32_t hi = tiny ? 0u : (special ? 0x7FF80000u : (a >> 3) + (896u << 20));  // bias 127 -> 1023
-  return __hiloint2double(int((u & 0x80000000u) | hi), int(tiny ? 0u : (u << 29)));
-}
-
-__device__ __forceinline__ float d2f(double x) {
-  const uint32_t hi = uint32_t(__double2hiint(x)), lo = uint32_t(__double2loint(x)), a = hi & 0x7FFFFFFFu;
-  uint32_t m = ((a - 0x38000000u) << 3) | (lo >> 29);  // bias 1023 -> 127, top 23 mantissa bits
-  // round to nearest even on the 29 dropped bits: up if above half, or at half with m odd
-  m += (lo >> 28) & ((lo & 0x0FFFFFFFu ? 1u : 0u) | m) & 1u;
-  m = a < 0x38100000u ? 0u : (a >= 0x47F00000u ? 0x7FC00000u : m);
-  return __uint_as_float((hi & 0x80000000u) | m);
-}
 
 // index of (i, j) in the packed row-major upper triangle of a symmetric 5x5 matrix
 __host__ __device__ constexpr int S(int i, int j) { return i <= j ? i * (9 - i) / 2 + j : j * (9 - j) / 2 + i; }
@@ -110,88 +88,6 @@ __device__ __forceinline__ void reload_uvf(const double* __restrict__ g, uint32_
 
 __device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-}
-
-// ------------------------------------------------------------------ FP64 without the FP64 pipe's divides
-// A division or square root in FP64 is a sequence of 8 to 12 FP64 instructions, and an FP64 warp
-// instruction holds its SM partition for 64 cycles on GB300 (integer, FP32 and special-function
-// instructions: 1 to 4). The FP64 path's stepping therefore takes reciprocals and roots by
-// Newton-Raphson (or one third-order step, which cubes the relative error) from the special-function
-// unit's or an FP32 seed, and compares magnitudes as integers. Products that feed a sum are written
-// as fma() or __dmul_rn, so that every instantiation (register caps, lanes a track) rounds alike.
-
-// |x| <= lim and |x| < lim for lim >= 0: the bit patterns of non-negative doubles order like the
-// values, NaN above all (so a NaN x is neither).
-__device__ __forceinline__ bool abs_le(double x, double lim) {
-  return (__double_as_longlong(x) & 0x7fffffffffffffffll) <= __double_as_longlong(lim);
-}
-__device__ __forceinline__ bool abs_lt(double x, double lim) {
-  return (__double_as_longlong(x) & 0x7fffffffffffffffll) < __double_as_longlong(lim);
-}
-
-// 1/x of a normal x well inside the exponent range, within an ulp: the special-function seed (2^-20)
-// and one third-order step.
-__device__ __forceinline__ double rcp_nr(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
-// 1/sqrt(x) of a normal x > 0, within about an ulp, in the same way.
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(__dmul_rn(-x, y), y, 1.0);
-  return fma(__dmul_rn(y, e), fma(e, 0.375, 0.5), y);
-}
-
-// a . b with a fixed order of roundings
-__device__ __forceinline__ double dot3f(const double a[3], const double b[3]) {
-  return fma(a[2], b[2], fma(a[1], b[1], __dmul_rn(a[0], b[0])));
-}
-__device__ __forceinline__ void crossf(const double a[3], const double b[3], double o[3]) {
-  o[0] = fma(a[1], b[2], -__dmul_rn(a[2], b[1]));
-  o[1] = fma(a[2], b[0], -__dmul_rn(a[0], b[2]));
-  o[2] = fma(a[0], b[1], -__dmul_rn(a[1], b[0]));
-}
-
-// Natural logarithm of a positive normal x (table-driven, after P. T. P. Tang, ACM TOMS 16, 1990):
-// x = 2^e m, c ~ 1/m from the top 7 bits of m, ln x = e ln 2 - ln c + ln(1 + z) with z = m c - 1,
-// |z| < 2^-8, by its series through z^7 (truncation below 2^-66). 11 FP64 instructions against about
-// 25 of log(); within 1.1 ulp in the callers' ranges (results of magnitude 4 to 40). Others: log().
-struct LogTable {
-  double c[128], l[128];  // c, -ln c
-};
-constexpr LogTable make_log_table() {
-  LogTable t{};
-  for (int j = 0; j < 128; ++j) {
-    const double c = 256.0 / (257.0 + 2.0 * j);
-    // -ln c = 2 artanh((1 - c) / (1 + c))
-    const double u = (1.0 - c) / (1.0 + c), u2 = u * u;
-    double sum = 0.0;
-    for (int k = 41; k >= 1; k -= 2) sum = sum * u2 + 1.0 / k;
-    t.c[j] = c;
-    t.l[j] = 2.0 * u * sum;
-  }
-  return t;
-}
-__device__ const LogTable kLogTable = make_log_table();
-
-__device__ __forceinline__ double log_nr(double x) {
-  const uint32_t hi = uint32_t(__double2hiint(x));
-  if (hi - 0x00100000u >= 0x7fe00000u) return log(x);
-  const int e = int(hi >> 20) - 1023;
-  const uint32_t j = (hi >> 13) & 127u;
-  const double m = __hiloint2double(int((hi & 0x000fffffu) | 0x3ff00000u), __double2loint(x));
-  const double z = fma(m, __ldg(&kLogTable.c[j]), -1.0);
-  double p = fma(z, 1.0 / 7, -1.0 / 6);
-  p = fma(z, p, 0.2);
-  p = fma(z, p, -0.25);
-  p = fma(z, p, 1.0 / 3);
-  p = fma(z, p, -0.5);
-  p = fma(__dmul_rn(z, z), p, z);
-  return fma(f2d(float(e)), 0.693147180559945309417, __ldg(&kLogTable.l[j])) + p;
 }
 
 // ------------------------------------------------------------------ field policies
@@ -1537,37 +1433,39 @@ __device__ __forceinline__ uint32_t combine_with_seed(const FitArgs& a, uint32_t
 
 // ---- all-states mode: the forward pass stores what the backward RTS pass needs.
 // Filtered state of entry m into the all-states arrays (SoA [5][n_meas], [15][n_meas]); at
-// the first entry p holds the angles, later the direction is carried as sines and cosines.
+// the first entry p holds the angles, later the direction is carried as sines and cosines. (The
+// predicted angles could be the filtered ones less the update's increments, but the mixed path turns
+// the direction by FP32 sines: 5e-9 rad off. Each is an arc tangent of its own, by atan2_nr: with the
+// records' 16-byte stores the mixed kernel went from 1.36 to 1.24 ms for 100,000 tracks.)
 template <class U>
 __device__ __forceinline__ void store_filtered(const FitArgs& a, uint32_t m, const double p[5], const U C[15],
                                                bool first, double sph, double cph, double sth, double cth) {
   const size_t nm = size_t(a.n_meas);
   a.states_par[m] = p[0];
   a.states_par[nm + m] = p[1];
-  a.states_par[2 * nm + m] = first ? p[2] : atan2(sph, cph);
-  a.states_par[3 * nm + m] = first ? p[3] : atan2(sth, cth);
+  a.states_par[2 * nm + m] = first ? p[2] : atan2_nr(sph, cph);
+  a.states_par[3 * nm + m] = first ? p[3] : atan2_nr(sth, cth);
   a.states_par[4 * nm + m] = p[4];
 #pragma unroll
   for (int j = 0; j < 15; ++j) a.states_cov[size_t(j) * nm + m] = cov_to_d(C[j]);
 }
 
-// Predicted state, packed covariance and transport Jacobian (row-major) of entry m into the
-// workspace: 45 doubles an entry, entry-major (kStatesScratch).
+// Predicted state, packed covariance and rows 0..3 of the transport Jacobian (row 4 is e_4) of entry m
+// into the workspace: 40 doubles an entry, entry-major, in 16-byte stores.
 template <class U>
 __device__ __forceinline__ void store_predicted(const FitArgs& a, uint32_t m, const double p[5], const U C[15],
                                                 const U J[5][5], double sp2, double cp2, double st2, double ct2) {
-  double* w = a.states_scratch + size_t(m) * kStatesScratch;
-  w[0] = p[0];
-  w[1] = p[1];
-  w[2] = atan2(sp2, cp2);
-  w[3] = atan2(st2, ct2);
-  w[4] = p[4];
+  double2* w = reinterpret_cast<double2*>(a.states_scratch + size_t(m) * kStatesScratch);
+  w[0] = make_double2(p[0], p[1]);
+  w[1] = make_double2(atan2_nr(sp2, cp2), atan2_nr(st2, ct2));
+  w[2] = make_double2(p[4], cov_to_d(C[0]));
 #pragma unroll
-  for (int j = 0; j < 15; ++j) w[5 + j] = cov_to_d(C[j]);
+  for (int j = 0; j < 7; ++j) w[3 + j] = make_double2(cov_to_d(C[2 * j + 1]), cov_to_d(C[2 * j + 2]));
 #pragma unroll
-  for (int r = 0; r < 5; ++r)
-#pragma unroll
-    for (int c = 0; c < 5; ++c) w[20 + 5 * r + c] = cov_to_d(J[r][c]);
+  for (int j = 0; j < 10; ++j) {
+    const int e = 2 * j, f = 2 * j + 1;
+    w[10 + j] = make_double2(cov_to_d(J[e / 5][e % 5]), cov_to_d(J[f / 5][f % 5]));
+  }
 }
 
 template <int kPrec, int kMode, int kG, int kPlace, int kSmooth, bool kRoll, class F>

@@ -90,9 +90,9 @@ struct FitArgs {
   double* __restrict__ states_scratch;  // workspace: kStatesScratch doubles per entry
 };
 
-// Per entry for the backward RTS pass: predicted parameters (5), packed covariance (15) and the
-// transport Jacobian from the previous entry (25, row-major).
-constexpr int kStatesScratch = 45;
+// Per entry for the backward RTS pass: predicted parameters (5), packed covariance (15) and rows 0..3 of
+// the transport Jacobian from the previous entry (20, row-major; row 4 is e_4), 16-byte aligned.
+constexpr int kStatesScratch = 40;
 
 constexpr int kMlpParams = TKF_MLP_PARAMS;
 constexpr int kMlpRecord = TKF_MLP_RECORD;
@@ -109,8 +109,9 @@ struct Workspace {
 size_t workspace_bytes(uint32_t n_tracks, bool learned, uint64_t states_entries = 0);
 Workspace carve_workspace(void* base, uint32_t n_tracks, bool learned, uint64_t states_entries = 0);
 // Backward RTS pass of the all-states output (tkf_states.cu), after the fit on the same stream;
-// perm: the fit's track order.
-cudaError_t launch_smooth_states(const FitArgs& a, const uint32_t* perm, cudaStream_t stream);
+// perm: the fit's track order; axial: a field along z (row 3 of every Jacobian is (0, 0, 0, J33, J34));
+// fp64: the states of the FP64 fit.
+cudaError_t launch_smooth_states(const FitArgs& a, const uint32_t* perm, bool axial, bool fp64, cudaStream_t stream);
 cudaError_t launch_propose_start(const FitArgs& a, const FieldDev& f, float* h0, cudaStream_t stream);
 
 // Seed parameter estimation (tkf_seed.cu): one thread per track, outputs in the fit's seed layout.

@@ -150,7 +150,9 @@ cudaError_t launch_fit(const FitArgs& a, const FieldDev& f, int precision, const
                                     : launch_fit_fp64(b, f, mode, ws.perm, ws.counter, shape, stream);
   if (e != cudaSuccess) return e;
   if (timing && (e = cudaEventRecord(timing[1], stream)) != cudaSuccess) return e;
-  if (mode == 3) e = launch_smooth_states(b, ws.perm, stream);  // backward RTS over the stored states
+  if (mode == 3)  // backward RTS over the stored states
+    e = launch_smooth_states(b, ws.perm, f.kind == TKF_FIELD_UNIFORM && f.b[0] == 0.0 && f.b[1] == 0.0,
+                             precision == TKF_FP64, stream);
   return e;
 }
 

@@ -27,43 +27,6 @@ __device__ __forceinline__ double rsqrt_pos(double x) { return x > 1e-290 && x <
 // from the arc and dz instead of a sine, arc tangents from a table (atan2_nr), and the Highland factor of
 // a surface from its record (computed once when the geometry is created). 600,000 tracks: 351 -> 236 us.
 
-// atan2(y, x) (table-driven, after P. T. P. Tang, ACM TOMS 16, 1990): with t = min / max of |x|, |y| and
-// k ~ 16 t, atan t = atan(k / 16) + atan(d), d = (min - k/16 max) / (max + k/16 min), |d| < 2^-4.9, by its
-// series through d^11 (truncation below 2^-61 relative). 20 FP64 instructions against more than 50 of
-// atan2(), within 1.9 ulp (CUDA's atan2: 2). Outside the FP32 range, and where an argument is not finite: atan2().
-__device__ const double kAtan16[17] = {  // atan(k / 16)
-    0.0, 0.06241880999595735, 0.12435499454676144, 0.18534794999569476, 0.24497866312686414, 0.3028848683749714,
-    0.35877067027057225, 0.4124104415973873, 0.4636476090008061, 0.5123894603107377, 0.5585993153435624,
-    0.6022873461349642, 0.6435011087932844, 0.6823165548747481, 0.7188299996216245, 0.7531512809621944,
-    0.7853981633974483};
-
-__device__ __forceinline__ double atan2_nr(double y, double x) {
-  const float xf = fabsf(d2f(x)), yf = fabsf(d2f(y));
-  const float big = fmaxf(xf, yf);
-  if (!(xf < 1e30f && yf < 1e30f && big > 1e-30f)) return atan2(y, x);
-  const bool steep = abs_lt(x, fabs(y));
-  const double mn = steep ? fabs(x) : fabs(y), mx = steep ? fabs(y) : fabs(x);
-  const float kf = rintf(__fdividef(fminf(xf, yf), big) * 16.0f);
-  const double c = f2d(kf * 0.0625f), num = fma(-c, mx, mn), den = fma(c, mn, mx);
-  double inv;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(inv) : "d"(den));
-  inv = fma(inv, fma(-den, inv, 1.0), inv);  // 2^-40; the quotient's remainder gives the rest
-  double d = __dmul_rn(num, inv);
-  d = fma(fma(-d, den, num), inv, d);
-  const double e = __dmul_rn(d, d);
-  double p = fma(e, -1.0 / 11, 1.0 / 9);
-  p = fma(e, p, -1.0 / 7);
-  p = fma(e, p, 0.2);
-  p = fma(e, p, -1.0 / 3);
-  const double t = __ldg(&kAtan16[int(kf)]) + fma(__dmul_rn(d, e), p, d);
-  // t, pi/2 - t, pi/2 + t or pi - t, with the part of pi below its double
-  constexpr double kPiLo = 1.2246467991473532e-16;
-  const bool back = __double2hiint(x) < 0;
-  const double base = steep ? 0.5 * kPi : (back ? kPi : 0.0), lo = steep ? 0.5 * kPiLo : (back ? kPiLo : 0.0);
-  const double r = base + ((steep != back ? -t : t) + lo);
-  return copysign(r, y);
-}
-
 // phi, theta and q/p at point r1 of the helix (axis z, field bz) through r1, r2, r3 in the
 // order of travel; also 1/radius (0 without curvature) and sin(theta). Returns
 // TKF_SEED_NO_CURVATURE for collinear points or bz = 0.
