@@ -48,6 +48,12 @@ __device__ __forceinline__ bool abs_lt(double x, double lim) {
   return (__double_as_longlong(x) & 0x7fffffffffffffffll) < __double_as_longlong(lim);
 }
 
+// x > 0, as an integer test in FP64 (false for NaN)
+__device__ __forceinline__ bool positive(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+
 // 1/x of a normal x well inside the exponent range, within an ulp: the special-function seed (2^-20)
 // and one third-order step.
 __device__ __forceinline__ double rcp_nr(double x) {
