@@ -2070,6 +2070,10 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
     fit_persistent_kernel(FitArgs a, F fld, const uint32_t* __restrict__ perm, uint32_t* __restrict__ counter,
                           uint32_t tpw) {
   constexpr int kPlace = kPrec == 2 ? 0 : reg_state_place(kRegs);
+  // the column loops stay rolled at 64 registers, and in the mixed path's field map at 128 too, whose code is
+  // the longest (three lookups a step; 100,000 map muons 1.39 -> 1.36 ms, 300,000 3.70 -> 3.55, two-filter
+  // 200,000 4.66 -> 4.54)
+  constexpr bool kRoll = kRegs == 64 || (kRegs == 128 && kPrec == 1 && !F::kUniform);
   extern __shared__ double smem_state[];
   SmootherStore<kPlace, typename CovType<kPrec>::type> st{};
   if constexpr (kPlace != 0) st.s = smem_state + threadIdx.x * state_doubles(kPlace);
@@ -2083,7 +2087,7 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
     if (base >= a.n_tracks) break;
     const uint32_t j = base + g;
     if (g < tpw && j < a.n_tracks)
-      fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRegs == 64>(a, fld, perm[j], st, gl, gmask);
+      fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll>(a, fld, perm[j], st, gl, gmask);
   }
 }
 
