@@ -1132,7 +1132,7 @@ tkf_status tkf_mlp_forward(tkf_context ctx, const float* params, const float* x,
 namespace {
 
 constexpr uint32_t kNoallocMaxTracks = TKF_NOALLOC_MAX_TRACKS;
-constexpr size_t kNoallocWords = 1 + 1024 + 2 * size_t(kNoallocMaxTracks) + 64;
+constexpr size_t kNoallocWords = 1 + tkf::kOrderBins + 2 * size_t(kNoallocMaxTracks) + 64;
 
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kNoallocWords];
 

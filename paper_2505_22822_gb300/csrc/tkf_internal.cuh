@@ -97,6 +97,9 @@ constexpr int kStatesScratch = 40;
 constexpr int kMlpParams = TKF_MLP_PARAMS;
 constexpr int kMlpRecord = TKF_MLP_RECORD;
 
+// Bins of the track ordering's keys (tkf_order.cu).
+constexpr int kOrderBins = 8192;
+
 // Scratch of one fit launch: work counter, key histogram, sort keys, track permutation.
 struct Workspace {
   uint32_t* counter = nullptr;

@@ -42,3 +42,14 @@ def test_both_sides_of_every_line(case, precision, smoother, per_sm, extra):
     torch.cuda.synchronize()
     for k in ("par", "cov", "chi2", "ndf", "status", "steps"):
         np.testing.assert_array_equal(getattr(a, k).cpu().numpy(), getattr(f, k).cpu().numpy(), err_msg=k)
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 8191, 8192, 8193, 9216])
+def test_ordering_by_one_block_or_many(case, n):
+    """Up to 8,192 tracks one block orders the batch; every track is fitted once on both sides of that."""
+    ctx, _, geo, fld, b, mass = case
+    opts = tkf.Options(precision=tkf.MIXED, mass=mass)
+    a, f = tkf.fit(ctx, geo, fld, _first(b, n), opts), tkf.fit(ctx, geo, fld, _first(b, 10_000), opts)
+    torch.cuda.synchronize()
+    for k in ("par", "cov", "chi2", "ndf", "status", "steps"):
+        np.testing.assert_array_equal(getattr(a, k).cpu().numpy(), getattr(f, k)[..., :n].cpu().numpy(), err_msg=k)
