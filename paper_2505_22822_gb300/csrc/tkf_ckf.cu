@@ -489,11 +489,16 @@ __device__ int navigate(const CkfArgs& a, int cur, const double x[3], const doub
   return best;
 }
 
-// From a branch's filtered state on its surface: material, navigation, RKN propagation and
-// covariance transport to the next module; returns its id (-1: none ahead, or stopped).
+constexpr int kCkfTries = 4;  // modules a branch may try on its way to the next one
+constexpr int kRetry = -3;    // predict: the module was not reached inside its extents
+
+// From a branch's filtered state on its surface: material, navigation (without the modules already
+// tried), RKN propagation and covariance transport to the next module; returns its id, or -1 if none lies
+// ahead or the particle stopped. A module that the propagation misses is added to skip; the next one is
+// tried at once, or (once) left to a later call by returning kRetry. -1 after kCkfTries.
 template <bool kMixed, class F>
-__device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, const CkfBranch& br, double pp[5],
-                       double pdir[4], double Cp[15], double& h_ctrl) {
+__device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, const CkfBranch& br, uint32_t* skip,
+                       uint32_t& nskip, bool once, double pp[5], double pdir[4], double Cp[15], double& h_ctrl) {
   Surf sc;
   load_surf(a.surf, uint32_t(br.sid), sc);
   const double sph = br.dir[0], cph = br.dir[1], sth = br.dir[2], cth = br.dir[3];
@@ -517,10 +522,8 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
   double kc[3];
   crossf(T0, B, kc);
   for (int j = 0; j < 3; ++j) kc[j] *= kl;
-  uint32_t skip[4];
-  int nskip = 0;
-  for (int tries = 0; tries < 4; ++tries) {
-    const int m = navigate(a, br.sid, x, T0, kc, bend, skip, nskip, nt);
+  for (;;) {
+    const int m = navigate(a, br.sid, x, T0, kc, bend, skip, int(nskip), nt);
     if (m < 0) return -1;
     Surf s;
     load_surf(a.surf, uint32_t(m), s);
@@ -538,7 +541,9 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
       double hu, hv;
       module_half(a, nt, uint32_t(m), hu, hv);
       if ((st & ~TKF_TRACK_OUT_OF_FIELD) || fabs(dot3(s.u, d)) > hu || fabs(dot3(s.v, d)) > hv) {
+        if (nskip + 1 >= uint32_t(kCkfTries)) return -1;
         skip[nskip++] = uint32_t(m);
+        if (once) return kRetry;
         continue;
       }
       // bound parameters (FP64 from the anchors) and the transport Jacobian in FP32
@@ -587,7 +592,9 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
       double hu, hv;
       module_half(a, nt, uint32_t(m), hu, hv);
       if (st || fabs(l0) > hu || fabs(l1) > hv) {
+        if (nskip + 1 >= uint32_t(kCkfTries)) return -1;
         skip[nskip++] = uint32_t(m);
+        if (once) return kRetry;
         continue;
       }
       const AxialTarget t = axial_target(s, T, __dmul_rn(__dmul_rn(lam, kKappa), fld.bz));
@@ -632,7 +639,9 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
       double hu, hv;
       module_half(a, nt, uint32_t(m), hu, hv);
       if ((st & ~TKF_TRACK_OUT_OF_FIELD) || fabs(dot3(s.u, d)) > hu || fabs(dot3(s.v, d)) > hv) {
+        if (nskip + 1 >= uint32_t(kCkfTries)) return -1;
         skip[nskip++] = uint32_t(m);
+        if (once) return kRetry;
         continue;
       }
       // bound parameters and the transport Jacobian at the target (path correction)
@@ -668,7 +677,6 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
       return m;
     }
   }
-  return -1;
 }
 
 // predicted chi2 of a measurement (no update)
@@ -959,12 +967,18 @@ __global__ void __launch_bounds__(kCkfBlock) ckf_nav_kernel(const CkfArgs a, Nav
   for (uint32_t j = threadIdx.x; j < sizeof(NavTables) / 16; j += blockDim.x) dst[j] = src[j];
 }
 
-// Phase 1: the prediction of the branch at list entry k (beam slot g = t B + bi).
+// A branch to predict: list entry k and the modules that earlier tries missed.
+struct CkfItem {
+  uint32_t k, nskip, skip[kCkfTries - 1];
+};
+
+// Phase 1: the prediction of the branch at list entry it.k (beam slot g = t B + bi); true when, with
+// `once`, another try is due (it.skip has grown).
 template <bool kMixed, class F>
-__device__ __forceinline__ void predict_branch(const CkfArgs& a, const F& fld, const NavTables& nt, const CkfWork& w,
-                                               uint32_t k) {
+__device__ __forceinline__ bool predict_branch(const CkfArgs& a, const F& fld, const NavTables& nt, const CkfWork& w,
+                                               bool once, CkfItem& it) {
   const uint32_t B = a.beam;
-  const uint32_t g = w.list[k];  // a branch slot in the beam
+  const uint32_t g = w.list[it.k];  // a branch slot in the beam
   const uint32_t t = g / B, bi = g % B;
   const CkfSeed st = w.seeds[t];
   CkfPred& pr = w.pred[g];
@@ -975,37 +989,82 @@ __device__ __forceinline__ void predict_branch(const CkfArgs& a, const F& fld, c
     store_pred(pr, br.p, br.dir, br.C, br.h_ctrl);
   } else {
     double pp[5], pdir[4], Cp[15], h = br.h_ctrl;
-    target = br.n_entries >= a.max_entries ? -1 : predict<kMixed>(a, fld, nt, br, pp, pdir, Cp, h);
+    target = br.n_entries >= a.max_entries
+                 ? -1
+                 : predict<kMixed>(a, fld, nt, br, it.skip, it.nskip, once, pp, pdir, Cp, h);
+    if (target == kRetry) return true;
     if (target >= 0) store_pred(pr, pp, pdir, Cp, h);
   }
   pr.target = target;
+  return false;
 }
 
-// One wave of resident blocks: each copies the navigation tables once, then takes chunks of
-// blockDim.x list entries from a counter until the list is done (branches differ in their work,
-// so the chunks balance the blocks). No block waits on another.
-template <bool kMixed, class F>
+// One wave of resident blocks: each copies the navigation tables once, then takes chunks of list entries
+// from a counter until the list is done. No block waits on another.
+//
+// A tenth of the branches miss the module that the parabola pointed at and navigate again: with the tries
+// in a loop, nearly every warp runs a second round for two or three lanes. In mixed precision, on a list
+// that fills the blocks more than twice, missed branches wait in the block's queue instead, which is worked
+// off a block at a time (or when the list is done): 80,000 seeds of five events 12.7 -> 11.6 ms. On shorter
+// lists the rounds of the queue follow one another where the tries of different warps overlap (one event
+// of 10,000 seeds 4.0 against 4.5 ms), and in FP64 the repeated material costs as much as it saves (80,000
+// seeds 17.6 against 17.9).
+// The warps of a block stay in step, round by round: the kernel waits on instruction fetch, and warps at
+// the same place share it (a queue a warp, without the barriers, doubled those stalls: 13.2 ms).
+constexpr uint32_t kCkfQueue = 2 * kCkfBlock;  // fewer than a block's worth waiting, and a round's more
+template <bool kMixed, bool kQueue, class F>
 __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a, const F fld, CkfWork w) {
   __shared__ NavTables nt;
-  __shared__ uint32_t chunk;
-  const uint32_t count = *w.count;
-  if (blockIdx.x * blockDim.x >= count) return;  // more blocks than chunks: none for this one
+  __shared__ CkfItem queue[kQueue ? kCkfQueue : 1];
+  __shared__ uint32_t chunk, waiting;
+  const uint32_t count = *w.count, tid = threadIdx.x;
+  if (blockIdx.x * kCkfBlock >= count) return;  // more blocks than chunks: none for this one
   const uint4* src = reinterpret_cast<const uint4*>(w.nav);
   uint4* dst = reinterpret_cast<uint4*>(&nt);
-  for (uint32_t j = threadIdx.x; j < sizeof(NavTables) / 16; j += blockDim.x) dst[j] = src[j];
+  for (uint32_t j = tid; j < sizeof(NavTables) / 16; j += blockDim.x) dst[j] = src[j];
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     const bool ring_fit = a.n_rings <= uint32_t(kCkfMaxRings);
     nt.rings = ring_fit ? nt.ring : a.rings;
     nt.rings_f = ring_fit ? nt.ring_f : nullptr;
+    waiting = 0;
   }
-  for (;;) {
-    if (threadIdx.x == 0) chunk = atomicAdd(w.next, blockDim.x);
-    __syncthreads();  // (the first one also publishes the ring pointers)
-    const uint32_t b0 = chunk;
-    __syncthreads();
-    if (b0 >= count) break;
-    if (b0 + threadIdx.x < count) predict_branch<kMixed>(a, fld, nt, w, b0 + threadIdx.x);
+  if constexpr (!kQueue) {
+    for (;;) {
+      if (tid == 0) chunk = atomicAdd(w.next, uint32_t(kCkfBlock));
+      __syncthreads();  // (the first one also publishes the ring pointers)
+      const uint32_t base = chunk;
+      __syncthreads();
+      if (base >= count) break;
+      CkfItem it{base + tid, 0u, {0u, 0u, 0u}};
+      if (it.k < count) predict_branch<kMixed>(a, fld, nt, w, false, it);
+    }
+  } else {
+    const bool once = count > 2u * gridDim.x * kCkfBlock;
+    for (bool more = true;;) {
+      __syncthreads();  // the queue of the last round (at first: its emptiness and the ring pointers)
+      const uint32_t left = waiting;
+      const bool drain = left >= uint32_t(kCkfBlock) || (!more && left > 0);
+      if (!drain && !more) break;
+      CkfItem it{0u, 0u, {0u, 0u, 0u}};
+      bool mine;
+      if (drain) {  // the queue's last entries
+        const uint32_t take = left < uint32_t(kCkfBlock) ? left : uint32_t(kCkfBlock);
+        mine = tid < take;
+        if (mine) it = queue[left - take + tid];
+        __syncthreads();
+        if (tid == 0) waiting = left - take;
+      } else {
+        if (tid == 0) chunk = atomicAdd(w.next, uint32_t(kCkfBlock));
+        __syncthreads();
+        const uint32_t base = chunk;
+        more = base < count;
+        mine = base + tid < count;
+        it.k = base + tid;
+      }
+      __syncthreads();
+      if (mine && predict_branch<kMixed>(a, fld, nt, w, once, it)) queue[atomicAdd(&waiting, 1u)] = it;
+    }
   }
 }
 
@@ -1249,21 +1308,20 @@ cudaError_t launch_ckf(const CkfArgs& a_in, const F& fld, cudaStream_t stream) {
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  e = a.mixed ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ckf_predict_kernel<true, F>, kCkfBlock, 0)
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ckf_predict_kernel<false, F>, kCkfBlock, 0);
+  auto* predict = a.mixed ? ckf_predict_kernel<true, false, F> : ckf_predict_kernel<false, false, F>;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, predict, kCkfBlock, 0);
   if (e != cudaSuccess) return e;
   const unsigned wave = unsigned(sms > 0 ? sms : 1) * unsigned(per_sm > 0 ? per_sm : 1);
   const unsigned gp = gb < wave ? gb : wave;
+  // beams that can fill the wave more than twice: missed branches wait in the blocks' queues
+  if (a.mixed && size_t(a.n_seeds) * a.beam > size_t(2) * wave * kCkfBlock) predict = ckf_predict_kernel<true, true, F>;
   if ((e = cudaMemsetAsync(w.count, 0, 2 * sizeof(uint32_t), stream)) != cudaSuccess) return e;
   ckf_nav_kernel<<<1, kCkfBlock, 0, stream>>>(a, nav);
   ckf_init_kernel<<<gs, kCkfBlock, 0, stream>>>(a, w);
   // every step adds an entry to each surviving branch: at most max_entries + 2 steps
   const uint32_t n_steps = ckf_steps(a.max_entries);
   for (uint32_t step = 0; step < n_steps; ++step) {
-    if (a.mixed)
-      ckf_predict_kernel<true><<<gp, kCkfBlock, 0, stream>>>(a, fld, w);
-    else
-      ckf_predict_kernel<false><<<gp, kCkfBlock, 0, stream>>>(a, fld, w);
+    predict<<<gp, kCkfBlock, 0, stream>>>(a, fld, w);
     ckf_gate_kernel<<<gb, kCkfBlock, 0, stream>>>(a, w);
     if ((e = cudaMemsetAsync(w.count, 0, 2 * sizeof(uint32_t), stream)) != cudaSuccess) return e;
     ckf_beam_kernel<<<gs, kCkfBlock, 0, stream>>>(a, w, step, step + 1 == n_steps ? 1u : 0u);
