@@ -21,6 +21,8 @@
 
 #include <math.h>
 
+#include <algorithm>
+
 #include "tkf_fp64.cuh"
 #include "tkf_internal.cuh"
 
@@ -1489,10 +1491,11 @@ __device__ __forceinline__ void store_predicted(const FitArgs& a, uint32_t m, co
   }
 }
 
-template <int kPrec, int kMode, int kG, int kPlace, int kSmooth, bool kRoll, class F>
+// kStep: every lane of the block calls this together, lanes that are not live only keep step
+template <int kPrec, int kMode, int kG, int kPlace, int kSmooth, bool kRoll, bool kStep, class F>
 __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
-                          SmootherStore<kPlace, typename CovType<kPrec>::type> st, uint32_t gl = 0,
-                          uint32_t gmask = 0xffffffffu) {
+                          SmootherStore<kPlace, typename CovType<kPrec>::type> st, uint32_t gl, uint32_t gmask,
+                          bool live, int n_max) {
   constexpr bool kMixed = kPrec != 0;
   static_assert(kG == 1 || kMode != kRecord, "record capture runs one lane per track");
   static_assert(kSmooth == 0 || (kG == 1 && kMode != kRecord), "the two-filter smoother runs one lane a track");
@@ -1521,15 +1524,19 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       M += (sid & TKF_SID_NO_MEASUREMENT) ? 0 : 1;
     }
   }
-  if (M == 0 && status == 0) {  // nothing to fit (no entry, or no measurement): the seed
-    if (!writer) return;
+  const bool seed_only = M == 0 && status == 0;  // nothing to fit (no entry, or no measurement): the seed
+  if (seed_only && writer && (!kStep || live)) {
     for (int j = 0; j < 5; ++j) a.par[size_t(j) * n + i] = p[j];
     for (int j = 0; j < 15; ++j) a.cov[size_t(j) * n + i] = cov_to_d(C[j]);
     a.chi2[i] = 0.0;
     a.ndf[i] = 0;
     a.status[i] = TKF_TRACK_TOO_FEW_HITS;
     if (a.steps) { a.steps[i] = 0; a.steps[n + i] = 0; }
-    return;
+  }
+  if constexpr (kStep) {
+    if (seed_only || !live) N = 0;  // the lane only keeps step
+  } else {
+    if (seed_only) return;
   }
   if (status == 0) {
     bool fin = true;
@@ -1569,10 +1576,17 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
   for (int pass = 0; pass < kPasses; ++pass) {
   const bool bwd = pass == 1;
   if (bwd) {
-    if (status & kFatal) break;
-    reverse_for_backward(p, C, sph, cph, cth, U(a.backward_inflation));
+    if (!kStep && (status & kFatal)) break;
+    if (!(status & kFatal)) reverse_for_backward(p, C, sph, cph, cth, U(a.backward_inflation));
   }
-  for (int ent = 0; ent < N && !(status & kFatal); ++ent) {
+  // in step, every lane of the block passes n_max barriers: its own entries first, then none
+  for (int ent = 0; kStep ? ent < n_max : (ent < N && !(status & kFatal)); ++ent) {
+    if constexpr (kStep) __syncthreads();
+    if (!kStep || (ent < N && !(status & kFatal))) do {
+// a fatal status ends the track: out of the loop, or past the rest of the entry to the next barrier
+#define TKF_LEAVE_ENTRY      \
+  if constexpr (kStep) break; \
+  else goto entries_done
     const int k = bwd ? N - 1 - ent : ent;
     const uint32_t m = b0 + k;
     Surf s;
@@ -1596,14 +1610,14 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       double lam = p[4], th0sq = 0.0;
       if (!bwd) {
         status |= material(sp, a.mat, a.opt, T, lam, th0sq);
-        if (status & kFatal) break;
+        if (status & kFatal) TKF_LEAVE_ENTRY;
       }
       double rho[3], D[3] = {0.0, 0.0, 0.0}, dr[2] = {0.0, 0.0}, dT[2] = {0.0, 0.0}, path = 0.0;
 #pragma unroll
       for (int j = 0; j < 3; ++j) rho[j] = s.c[j] - fma(p[1], sp.v[j], fma(p[0], sp.u[j], sp.c[j]));
       status |= propagate_z<kMode == kRecord ? kRecord : kPlain>(fld, a.opt, s, rho, D, T, lam, dr, dT, path, h_ctrl,
                                                                  attempts, rejected, learn);
-      if (status & kFatal) break;
+      if (status & kFatal) TKF_LEAVE_ENTRY;
       // ---- bound parameters at the target and the transport Jacobian (path correction)
       const AxialTarget t = axial_target(s, T, __dmul_rn(__dmul_rn(lam, kKappa), fld.bz));
       sp2 = t.sp2;
@@ -1658,7 +1672,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       double lam = p[4], th0sq = 0.0;
       if (!bwd) {
         status |= material(sp, a.mat, a.opt, T, lam, th0sq);
-        if (status & kFatal) break;
+        if (status & kFatal) TKF_LEAVE_ENTRY;
       }
       double r[3];
       for (int j = 0; j < 3; ++j) r[j] = sp.c[j] + p[0] * sp.u[j] + p[1] * sp.v[j];
@@ -1676,7 +1690,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       double kend[3];
       status |= propagate<kMode == kRecord ? kRecord : kPlain, kCols>(fld, a.opt, s, r, T, lam, dr, dT, qcol, h_ctrl,
                                                                       attempts, rejected, kend, learn);
-      if (status & kFatal) break;
+      if (status & kFatal) TKF_LEAVE_ENTRY;
       // ---- bound parameters at the target and the transport Jacobian (path correction)
       double inv_st, nrm;
       bound_direction(T, sp2, cp2, st2, ct2, inv_st, nrm);
@@ -1725,7 +1739,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       float th0sq = 0.0f;
       if (!bwd) {
         status |= material_mixed(sp, a.mat, a.opt, Tm, lam, th0sq);
-        if (status & kFatal) break;
+        if (status & kFatal) TKF_LEAVE_ENTRY;
       }
       double T[3] = {sth * cph, sth * sph, cth};
       double r[3];
@@ -1754,7 +1768,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       float kend[3];
       status |= propagate_mixed<kMode == kRecord ? kRecord : kPlain, kCols, F, kRoll>(
           fld, a.opt, s, nf, r, T, lam, dr, dT, qcol, h_ctrl_f, attempts, rejected, kend, learn);
-      if (status & kFatal) break;
+      if (status & kFatal) TKF_LEAVE_ENTRY;
       // direction at the target in FP64 from FP32-seeded Newton steps (relative error ~1e-14)
       const double t2 = dot3(T, T), e2 = t2 - 1.0;
       const double inv_norm = abs_lt(e2, 1e-4) ? 1.0 - e2 * (0.5 - 0.375 * e2) : 1.0 / sqrt(t2);
@@ -1826,7 +1840,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       }
       if (bwd) {  // the material of the surface reached, crossed against the flight direction
         status |= arrival_material<kPrec>(a, s, sp2, cp2, st2, ct2, p, C);
-        if (status & kFatal) break;
+        if (status & kFatal) TKF_LEAVE_ENTRY;
       }
       if constexpr (kMode == kStates) store_predicted(a, m, p, C, J, sp2, cp2, st2, ct2);
       // ---- smoother: R = P J^T (in place; J row 4 is e_4); the row loop stays rolled in the
@@ -1895,14 +1909,14 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
     if (measured) {
       // the track's chi2 is the forward filter's; the backward filter's goes to chi2_bwd
       status |= kalman_update<kG>(a, m, p, C, K, Si00, Si01, Si11, r0, r1, bwd ? chi2_bwd : chi2, gl, gmask);
-      if (status & kFatal) break;
+      if (status & kFatal) TKF_LEAVE_ENTRY;
     }  // measured
     if (!bwd && k == 0) {
       if (p[2] > kPi) p[2] -= 2.0 * kPi;
       if (p[2] <= -kPi) p[2] += 2.0 * kPi;
       if (!(p[3] > 0.0 && p[3] < kPi)) {
         status |= TKF_TRACK_NON_FINITE;
-        break;
+        TKF_LEAVE_ENTRY;
       }
       sincos(p[2], &sph, &cph);
       sincos(p[3], &sth, &cth);
@@ -1931,7 +1945,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       // filtered direction: predicted angles plus the update's increments p[2], p[3]
       if (!turn_direction<kMixed>(p, sp2, cp2, st2, ct2, sph, cph, sth, cth)) {  // theta left (0, pi)
         status |= TKF_TRACK_NON_FINITE;
-        break;
+        TKF_LEAVE_ENTRY;
       }
       // W = R H^T S^-1; p_0|N += W r; C_0|N -= W (R H^T)^T; P = R - R H^T K^T
       if constexpr (kSmooth == 1) {
@@ -1982,8 +1996,14 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
     if constexpr (kMode == kStates) store_filtered(a, m, p, C, k == 0, sph, cph, sth, cth);
     if constexpr (!kMixed) sp = s;
     sid_prev = sid;
+    } while (false);
+#undef TKF_LEAVE_ENTRY
   }
+  [[maybe_unused]] entries_done:;
   }  // passes
+  if constexpr (kStep) {
+    if (seed_only || !live) return;
+  }
   if constexpr (kSmooth == 1) {
     if (!(status & kFatal)) status |= combine_with_seed(a, i, p, C, sph, cph, sth, cth, st);
   }
@@ -2063,6 +2083,21 @@ __host__ __device__ constexpr int reg_min_blocks(int regs) { return regs >= 255 
 // warps would take the L1 capacity those spills need: launch +6 %).
 __host__ __device__ constexpr int reg_state_place(int regs) { return regs == 128 ? 2 : 0; }
 
+// Fits whose block passes its entries in step, with one barrier an entry: the mixed fit at one lane a track. Its
+// entry is a long stretch of straight code, and waiting for instructions was its first stall (in the field map 8.8
+// warps an issue): warps that run the same stretch together share each fetch. The block takes tpw tracks a warp at
+// once and every lane passes as many barriers as its longest track has entries; the ordering by length keeps
+// the idle ones few. 128-thread blocks, ms without / with, at 128 and at 255 registers:
+//   uniform field 200,000 tracks 1.80 / 1.72, 1.84 / 1.73, learned 600,000 5.20 / 4.98, 5.49 / 4.99;
+//   field map 300,000 3.50 / 3.12, 3.93 / 3.21, 100,000 1.34 / 1.25, 1.49 / 1.24;
+//   two-filter 200,000 2.90 / 2.47, 2.92 / 2.49, in the field map 4.40 / 3.27, 4.67 / 3.27.
+// Blocks of 64 and 256 threads gain less (map 300,000 3.47 both). Left alone: 64 registers, which wait for their
+// spilled state (map 100,000 1.54 / 1.74), the all-states mode (100,000 2.14 / 2.15) and FP64, bound by its
+// pipe (600,000 10.13 / 10.04; map 50,000 3.77 / 3.92).
+__host__ __device__ constexpr bool in_step(int prec, int mode, int regs, int group) {
+  return prec == 1 && regs != 64 && group == 1 && (mode == kPlain || mode == kLearned);
+}
+
 // kG lanes a track (1, or 4 for the group-per-track mapping): a warp takes tpw <= 32 / kG tracks
 // at a time, lanes g kG .. g kG + kG - 1 fit track base + g together.
 template <int kPrec, int kMode, int kRegs, int kG, int kSmooth, class F>
@@ -2070,24 +2105,48 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
     fit_persistent_kernel(FitArgs a, F fld, const uint32_t* __restrict__ perm, uint32_t* __restrict__ counter,
                           uint32_t tpw) {
   constexpr int kPlace = kPrec == 2 ? 0 : reg_state_place(kRegs);
-  // the column loops stay rolled at 64 registers, and in the mixed path's field map at 128 too, whose code is
-  // the longest (three lookups a step; 100,000 map muons 1.39 -> 1.36 ms, 300,000 3.70 -> 3.55, two-filter
-  // 200,000 4.66 -> 4.54)
-  constexpr bool kRoll = kRegs == 64 || (kRegs == 128 && kPrec == 1 && !F::kUniform);
+  // the column loops stay rolled at 64 registers, and out of step in the mixed path's field map at 128 too, whose
+  // code is the longest (three lookups a step; 100,000 map muons 1.39 -> 1.36 ms); in step the unrolled loops
+  // are as fast or faster (100,000 1.30 -> 1.25, two-filter 200,000 3.39 -> 3.27)
+  constexpr bool kRoll =
+      kRegs == 64 || (kRegs == 128 && kPrec == 1 && !F::kUniform && !in_step(kPrec, kMode, kRegs, kG));
   extern __shared__ double smem_state[];
   SmootherStore<kPlace, typename CovType<kPrec>::type> st{};
   if constexpr (kPlace != 0) st.s = smem_state + threadIdx.x * state_doubles(kPlace);
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t g = lane / kG, gl = lane % kG;
   const uint32_t gmask = kG == 1 ? 0xffffffffu : ((1u << kG) - 1u) << (g * kG);
-  for (;;) {
-    uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(counter, tpw);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= a.n_tracks) break;
-    const uint32_t j = base + g;
-    if (g < tpw && j < a.n_tracks)
-      fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll>(a, fld, perm[j], st, gl, gmask);
+  if constexpr (in_step(kPrec, kMode, kRegs, kG)) {
+    __shared__ uint32_t next;
+    __shared__ int longest;
+    const uint32_t first = (threadIdx.x >> 5) * tpw + g;  // this lane's track of the block's share
+    for (;;) {
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        next = atomicAdd(counter, tpw * (blockDim.x >> 5));
+        longest = 0;
+      }
+      __syncthreads();
+      const uint32_t base = next;
+      if (base >= a.n_tracks) break;
+      const uint32_t j = base + first;
+      const bool live = g < tpw && j < a.n_tracks;
+      const uint32_t i = perm[live ? j : base];
+      const uint32_t b0 = a.offsets[i], b1 = a.offsets[i + 1];
+      if (b1 >= b0 && b1 <= a.n_meas) atomicMax(&longest, int(b1 - b0));
+      __syncthreads();
+      fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll, true>(a, fld, i, st, gl, gmask, live, longest);
+    }
+  } else {
+    for (;;) {
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(counter, tpw);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (base >= a.n_tracks) break;
+      const uint32_t j = base + g;
+      if (g < tpw && j < a.n_tracks)
+        fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll, false>(a, fld, perm[j], st, gl, gmask, true, 0);
+    }
   }
 }
 
@@ -2421,6 +2480,11 @@ cudaError_t launch_persistent(const FitArgs& a, const F& fld, const uint32_t* pe
   if (shape.threads > reg_block_threads(kRegs) || shape.tracks_per_warp * kG > 32) return cudaErrorInvalidConfiguration;
   const int place = kPrec == 2 ? 0 : reg_state_place(kRegs);
   const size_t smem = size_t(shape.threads) * state_doubles(place) * sizeof(double);
+  // no more blocks than shares of tracks: the block scheduler then spreads a small batch over the SMs, where the
+  // first blocks would take it all (mixed, 128 x 2 at 255 registers: 20,000 tracks 0.44 -> 0.37 ms, in the field map
+  // 0.65 -> 0.53, two-filter 10,000 0.64 -> 0.51)
+  const uint32_t share = uint32_t(shape.tracks_per_warp) * uint32_t(shape.threads / 32);
+  shape.blocks = std::min(shape.blocks, std::max(1, int((uint64_t(a.n_tracks) + share - 1) / share)));
   fit_persistent_kernel<kPrec, kMode, kRegs, kG, kSmooth>
       <<<shape.blocks, shape.threads, smem, stream>>>(a, fld, perm, counter, uint32_t(shape.tracks_per_warp));
   return cudaGetLastError();

@@ -54,12 +54,11 @@ std::array<int, 5> default_shape(int precision, bool record) {
 //   warps' tracks halved while every SM still gets a warp. FP64 3,000 tracks 0.87 -> 0.55 / 2.96 -> 2.31,
 //   12,500 1.03 -> 0.78 / 3.52 -> 2.60; mixed 3,000 0.36 -> 0.31 / 0.65 -> 0.44, 12,500 0.40 -> 0.40 /
 //   0.63 -> 0.61; at 20,000 one lane wins (mixed 0.46 against 0.55 / 0.65 against 0.88).
-// * mixed: the full register file while few warps are resident anyway (latency bound: no spills), up to 1.75
-//   waves (60,000 0.77 -> 0.68 / 1.06 -> 0.96; 80,000 0.86 against 0.90 / 1.14 against 1.23), then 128
-//   registers, and 64 once their 32 warps an SM are filled several times: RTS from 6 waves (200,000 1.94
-//   against 1.97 / 2.58 against 2.44; 300,000 2.87 -> 2.77 / 3.75 -> 3.43), two-filter from 3.5 (100,000
-//   1.72 against 1.95 / 2.59 against 2.75; 150,000 2.58 -> 2.36 / 3.74 -> 3.42). The all-states mode, which
-//   stores every entry, keeps the full register file (128: 100,000 tracks with holes 2.48 against 2.54).
+// * mixed: the full register file up to 4 waves, then 128 registers, whose 16 warps an SM hide more than their
+//   spills cost (in step; 255 / 128 registers: 60,000 map 0.83 / 1.00; 100,000 0.95 / 0.97, map 1.24 / 1.25,
+//   two-filter 1.35 / 1.37; 150,000 1.34 / 1.35, 1.69 / 1.65, 1.90 / 1.95; 200,000 1.73 / 1.72, two-filter
+//   2.49 / 2.47; 300,000 map 3.21 / 3.12). 64 registers are behind from 600,000 (5.00, learned 5.14 / 4.98) down. The
+//   all-states mode, which stores every entry, keeps the full register file (128: 100,000 tracks 2.15 / 2.22).
 // * FP64: the full register file (within 3 % of the best at every size: the FP64 pipe is the bottleneck).
 // * blocks of one warp, no more than there are chunks of tracks, while they are fewer than the resident
 //   warps: the block scheduler then spreads them evenly over the SMs (two-filter FP64 10,000 1.48 -> 1.28).
@@ -71,8 +70,8 @@ LaunchShape sized_shape(const FitArgs& a, int precision, uint32_t sms) {
     s.group = 4;
     s.tracks_per_warp = 8;
     while (s.tracks_per_warp > 1 && n <= uint32_t(s.tracks_per_warp / 2) * sms) s.tracks_per_warp /= 2;
-  } else if (precision == TKF_MIXED && !states && n > wave / 4 * 7) {
-    s.regs = n > (two_filter ? wave / 2 * 7 : wave * 6) ? 64 : 128;
+  } else if (precision == TKF_MIXED && !states && n > 4 * wave) {
+    s.regs = 128;
   }
   const uint32_t chunks = (n + s.tracks_per_warp - 1) / s.tracks_per_warp;
   const uint32_t per_sm = s.regs == 255 ? kResidentWarpsPerSm : 65536 / (s.regs * 32);  // warps
