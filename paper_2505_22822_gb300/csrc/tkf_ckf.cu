@@ -496,18 +496,23 @@ constexpr int kRetry = -3;    // predict: the module was not reached inside its 
 // tried), RKN propagation and covariance transport to the next module; returns its id, or -1 if none lies
 // ahead or the particle stopped. A module that the propagation misses is added to skip; the next one is
 // tried at once, or (once) left to a later call by returning kRetry. -1 after kCkfTries.
-template <bool kMixed, class F>
-__device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, const CkfBranch& br, uint32_t* skip,
-                       uint32_t& nskip, bool once, double pp[5], double pdir[4], double Cp[15], double& h_ctrl) {
+// kStep: every lane of the block makes the call, those without a branch to move (go = false) as well, and passes
+// two barriers, after the first try's navigation and after its propagation.
+template <bool kMixed, bool kStep, class F>
+__device__ int predict(bool go, const CkfArgs& a, const F& fld, const NavTables& nt, const CkfBranch& br,
+                       uint32_t* skip, uint32_t& nskip, bool once, double pp[5], double pdir[4], double Cp[15],
+                       double& h_ctrl) {
+  static_assert(kMixed || !kStep, "the FP64 prediction returns before the barriers");
   Surf sc;
-  load_surf(a.surf, uint32_t(br.sid), sc);
+  load_surf(a.surf, !kStep || go ? uint32_t(br.sid) : 0u, sc);
   const double sph = br.dir[0], cph = br.dir[1], sth = br.dir[2], cth = br.dir[3];
   const double T0[3] = {sth * cph, sth * sph, cth};
   double lam = br.p[4], th0sq;
   if constexpr (kMixed) {
     const float Tm[3] = {d2f(T0[0]), d2f(T0[1]), d2f(T0[2])};
     float th0sq_f;
-    if (material_mixed(sc, a.mat, a.opt, Tm, lam, th0sq_f) & ~(TKF_TRACK_OUT_OF_FIELD)) return -1;
+    if (material_mixed(sc, a.mat, a.opt, Tm, lam, th0sq_f) & ~(TKF_TRACK_OUT_OF_FIELD)) go = false;
+    if (!kStep && !go) return -1;
     th0sq = f2d(th0sq_f);
   } else {
     if (material(sc, a.mat, a.opt, T0, lam, th0sq) & ~(TKF_TRACK_OUT_OF_FIELD)) return -1;
@@ -522,11 +527,12 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
   double kc[3];
   crossf(T0, B, kc);
   for (int j = 0; j < 3; ++j) kc[j] *= kl;
-  for (;;) {
-    const int m = navigate(a, br.sid, x, T0, kc, bend, skip, int(nskip), nt);
-    if (m < 0) return -1;
+  for (bool first = true;; first = false) {
+    const int m = !kStep || go ? navigate(a, br.sid, x, T0, kc, bend, skip, int(nskip), nt) : -1;
+    if (kStep && first) __syncthreads();
+    if (!kStep && m < 0) return -1;
     Surf s;
-    load_surf(a.surf, uint32_t(m), s);
+    load_surf(a.surf, uint32_t(kStep && m < 0 ? 0 : m), s);
     if constexpr (kMixed) {
       double r[3] = {x[0], x[1], x[2]}, T[3] = {T0[0], T0[1], T0[2]};
       const float fsth = d2f(sth), fcth = d2f(cth), fsph = d2f(sph), fcph = d2f(cph);
@@ -535,8 +541,11 @@ __device__ int predict(const CkfArgs& a, const F& fld, const NavTables& nt, cons
       float kend[3], h = float(br.h_ctrl);
       uint32_t att = 0, rej = 0;
       StepLearn learn{nullptr, 0, nullptr, 0.0f};
-      const uint32_t st =
-          propagate_mixed<kPlain, 3>(fld, a.opt, s, s.nf, r, T, lam, dr, dT, 0.0f, h, att, rej, kend, learn);
+      uint32_t st = 0;
+      if (!kStep || m >= 0)
+        st = propagate_mixed<kPlain, 3>(fld, a.opt, s, s.nf, r, T, lam, dr, dT, 0.0f, h, att, rej, kend, learn);
+      if (kStep && first) __syncthreads();
+      if (kStep && m < 0) return -1;
       const double d[3] = {r[0] - s.c[0], r[1] - s.c[1], r[2] - s.c[2]};
       double hu, hv;
       module_half(a, nt, uint32_t(m), hu, hv);
@@ -973,27 +982,28 @@ struct CkfItem {
 };
 
 // Phase 1: the prediction of the branch at list entry it.k (beam slot g = t B + bi); true when, with
-// `once`, another try is due (it.skip has grown).
-template <bool kMixed, class F>
+// `once`, another try is due (it.skip has grown). kStep: every lane of the block makes the call, `mine` or not.
+template <bool kMixed, bool kStep, class F>
 __device__ __forceinline__ bool predict_branch(const CkfArgs& a, const F& fld, const NavTables& nt, const CkfWork& w,
-                                               bool once, CkfItem& it) {
+                                               bool once, CkfItem& it, bool mine) {
   const uint32_t B = a.beam;
-  const uint32_t g = w.list[it.k];  // a branch slot in the beam
+  const uint32_t g = w.list[!kStep || mine ? it.k : 0u];  // a branch slot in the beam
   const uint32_t t = g / B, bi = g % B;
   const CkfSeed st = w.seeds[t];
   CkfPred& pr = w.pred[g];
   const CkfBranch& br = seed_slots(w, t, B)[st.act[bi]];
-  int target;
-  if (st.first) {
-    target = int(a.seed_sid[a.perm[t]]);
-    store_pred(pr, br.p, br.dir, br.C, br.h_ctrl);
-  } else {
+  const bool seed = st.first, ended = br.n_entries >= a.max_entries;
+  int target = -1;
+  if (kStep || (!seed && !ended)) {
     double pp[5], pdir[4], Cp[15], h = br.h_ctrl;
-    target = br.n_entries >= a.max_entries
-                 ? -1
-                 : predict<kMixed>(a, fld, nt, br, it.skip, it.nskip, once, pp, pdir, Cp, h);
+    target = predict<kMixed, kStep>(mine && !seed && !ended, a, fld, nt, br, it.skip, it.nskip, once, pp, pdir, Cp, h);
     if (target == kRetry) return true;
     if (target >= 0) store_pred(pr, pp, pdir, Cp, h);
+  }
+  if (kStep && !mine) return false;
+  if (seed) {
+    target = int(a.seed_sid[a.perm[t]]);
+    store_pred(pr, br.p, br.dir, br.C, br.h_ctrl);
   }
   pr.target = target;
   return false;
@@ -1005,12 +1015,15 @@ __device__ __forceinline__ bool predict_branch(const CkfArgs& a, const F& fld, c
 // A tenth of the branches miss the module that the parabola pointed at and navigate again: with the tries
 // in a loop, nearly every warp runs a second round for two or three lanes. In mixed precision, on a list
 // that fills the blocks more than twice, missed branches wait in the block's queue instead, which is worked
-// off a block at a time (or when the list is done): 80,000 seeds of five events 12.7 -> 11.6 ms. On shorter
+// off a block at a time (or when the list is done): 80,000 seeds of five events 12.7 -> 11.7 ms. On shorter
 // lists the rounds of the queue follow one another where the tries of different warps overlap (one event
 // of 10,000 seeds 4.0 against 4.5 ms), and in FP64 the repeated material costs as much as it saves (80,000
 // seeds 17.6 against 17.9).
-// The warps of a block stay in step, round by round: the kernel waits on instruction fetch, and warps at
-// the same place share it (a queue a warp, without the barriers, doubled those stalls: 13.2 ms).
+// The queue's kernel waits on instruction fetch, and warps at the same place share it: the block passes each
+// round in step, and within it the navigation, the propagation and the transport (80,000 seeds of five events
+// 11.7 -> 10.6 ms, 40,000 of three in the field map 10.2 -> 8.6; a queue a warp, without any barrier, 13.2; two more
+// barriers in the navigation 10.5). The kernel without a queue keeps its warps apart: its few chunks run
+// one after another where others wait (3,000 seeds 3.16 against 3.28 ms). 128 registers, 4 blocks an SM: 11.1.
 constexpr uint32_t kCkfQueue = 2 * kCkfBlock;  // fewer than a block's worth waiting, and a round's more
 template <bool kMixed, bool kQueue, class F>
 __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a, const F fld, CkfWork w) {
@@ -1037,7 +1050,7 @@ __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a,
       __syncthreads();
       if (base >= count) break;
       CkfItem it{base + tid, 0u, {0u, 0u, 0u}};
-      if (it.k < count) predict_branch<kMixed>(a, fld, nt, w, false, it);
+      if (it.k < count) predict_branch<kMixed, false>(a, fld, nt, w, false, it, true);
     }
   } else {
     const bool once = count > 2u * gridDim.x * kCkfBlock;
@@ -1063,7 +1076,7 @@ __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a,
         it.k = base + tid;
       }
       __syncthreads();
-      if (mine && predict_branch<kMixed>(a, fld, nt, w, once, it)) queue[atomicAdd(&waiting, 1u)] = it;
+      if (predict_branch<kMixed, true>(a, fld, nt, w, once, it, mine)) queue[atomicAdd(&waiting, 1u)] = it;
     }
   }
 }
