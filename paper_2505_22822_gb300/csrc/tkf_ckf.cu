@@ -874,6 +874,7 @@ struct CkfWork {
   uint32_t* list;    // the branch slots (t B + bi) in the beam, for the next step's phases 1 and 2
   uint32_t* count;   // their number
   uint32_t* next;    // the prediction's next chunk of the list (reset with count)
+  uint32_t schedulers;  // warp schedulers of the device (4 an SM)
   CkfNode* nodes;    // per seed: ckf_steps(max_entries) x B history nodes
   const NavTables* nav;  // the navigation tables, built once a call (pointers fixed up per block)
 };
@@ -1013,7 +1014,7 @@ __device__ __forceinline__ bool predict_branch(const CkfArgs& a, const F& fld, c
   return false;
 }
 
-// One wave of resident blocks: each copies the navigation tables once, then takes chunks of list entries
+// One wave of resident blocks: each copies the navigation tables once, then takes shares of the list's entries
 // from a counter until the list is done. No block waits on another.
 //
 // A tenth of the branches miss the module that the parabola pointed at and navigate again: with the tries
@@ -1029,13 +1030,23 @@ __device__ __forceinline__ bool predict_branch(const CkfArgs& a, const F& fld, c
 // barriers in the navigation 10.5). The kernel without a queue keeps its warps apart: its few chunks run
 // one after another where others wait (3,000 seeds 3.16 against 3.28 ms). 128 registers, 4 blocks an SM: 11.1.
 constexpr uint32_t kCkfQueue = 2 * kCkfBlock;  // fewer than a block's worth waiting, and a round's more
+// Branches a warp takes: the whole list at once while it has no more than one warp for each of the device's warp
+// schedulers, with 4, 8 or 16 of 32 lanes. A warp runs the navigation and the tries of its lanes one after
+// another where they differ, so fewer lanes end sooner, on schedulers that had nothing to do (mixed, beam 3:
+// 500 seeds 2.58 -> 2.39 ms, 3,000 3.16 -> 3.01; FP64 600 3.48 -> 3.15, 3,000 4.31 -> 4.15; the last steps of 80,000
+// mixed seeds 10.19 -> 10.08). Two warps a scheduler gain less (FP64 3,000 4.21, 10,000 5.54 against 5.52).
+__device__ __forceinline__ uint32_t branches_a_warp(uint32_t count, uint32_t schedulers) {
+  return count <= 4u * schedulers ? 4u : (count <= 8u * schedulers ? 8u : (count <= 16u * schedulers ? 16u : 32u));
+}
 template <bool kMixed, bool kQueue, class F>
 __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a, const F fld, CkfWork w) {
   __shared__ NavTables nt;
   __shared__ CkfItem queue[kQueue ? kCkfQueue : 1];
   __shared__ uint32_t chunk, waiting;
   const uint32_t count = *w.count, tid = threadIdx.x;
-  if (blockIdx.x * kCkfBlock >= count) return;  // more blocks than chunks: none for this one
+  const uint32_t lanes = branches_a_warp(count, w.schedulers), share = lanes * (kCkfBlock / 32);
+  const uint32_t own = (tid & 31u) < lanes ? (tid >> 5) * lanes + (tid & 31u) : share;  // this lane's of the block's share
+  if (blockIdx.x * share >= count) return;  // more blocks than shares: none for this one
   const uint4* src = reinterpret_cast<const uint4*>(w.nav);
   uint4* dst = reinterpret_cast<uint4*>(&nt);
   for (uint32_t j = tid; j < sizeof(NavTables) / 16; j += blockDim.x) dst[j] = src[j];
@@ -1048,13 +1059,13 @@ __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a,
   }
   if constexpr (!kQueue) {
     for (;;) {
-      if (tid == 0) chunk = atomicAdd(w.next, uint32_t(kCkfBlock));
+      if (tid == 0) chunk = atomicAdd(w.next, share);
       __syncthreads();  // (the first one also publishes the ring pointers)
       const uint32_t base = chunk;
       __syncthreads();
       if (base >= count) break;
-      CkfItem it{base + tid, 0u, {0u, 0u, 0u}};
-      if (it.k < count) predict_branch<kMixed, false>(a, fld, nt, w, false, it, true);
+      CkfItem it{base + own, 0u, {0u, 0u, 0u}};
+      if (own < share && it.k < count) predict_branch<kMixed, false>(a, fld, nt, w, false, it, true);
     }
   } else {
     const bool once = count > 2u * gridDim.x * kCkfBlock;
@@ -1072,12 +1083,12 @@ __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a,
         __syncthreads();
         if (tid == 0) waiting = left - take;
       } else {
-        if (tid == 0) chunk = atomicAdd(w.next, uint32_t(kCkfBlock));
+        if (tid == 0) chunk = atomicAdd(w.next, share);
         __syncthreads();
         const uint32_t base = chunk;
         more = base < count;
-        mine = base + tid < count;
-        it.k = base + tid;
+        it.k = base + own;
+        mine = own < share && it.k < count;
       }
       __syncthreads();
       if (predict_branch<kMixed, true>(a, fld, nt, w, once, it, mine)) queue[atomicAdd(&waiting, 1u)] = it;
@@ -1333,7 +1344,8 @@ cudaError_t launch_ckf(const CkfArgs& a_in, const F& fld, cudaStream_t stream) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, predict, kCkfBlock, 0);
   if (e != cudaSuccess) return e;
   const unsigned wave = unsigned(sms > 0 ? sms : 1) * unsigned(per_sm > 0 ? per_sm : 1);
-  const unsigned gp = gb < wave ? gb : wave;
+  w.schedulers = 4u * unsigned(sms > 0 ? sms : 1);
+  const unsigned gp = 8u * gb < wave ? 8u * gb : wave;  // shares of a block: 128 down to 16 branches
   // beams that can fill the wave more than twice: missed branches wait in the blocks' queues
   if (a.mixed && size_t(a.n_seeds) * a.beam > size_t(2) * wave * kCkfBlock) predict = ckf_predict_kernel<true, true, F>;
   if ((e = cudaMemsetAsync(w.count, 0, 2 * sizeof(uint32_t), stream)) != cudaSuccess) return e;
