@@ -185,8 +185,12 @@ typedef struct tkf_fit_options {
    * variant capped at that many registers a thread, which keeps part of the per-track state in
    * local memory (at 128 the smoother state in shared memory) and holds more warps per SM. With
    * all four 0 the shape is the tuned one of this launch class when TKF_FIT_AUTOTUNE is set,
-   * else FP64: 128 threads x 2 blocks per SM, 255 registers; mixed: 128 x 4, 128 registers;
-   * 32 tracks per warp. An explicit part disables tuning; the other parts take defaults. */
+   * else one by the batch's size: four lanes a track up to 80 tracks an SM (RTS without all
+   * states), one lane a track and 255 registers above, blocks of one warp while they are fewer
+   * than the resident warps, 128 registers for the mixed fit beyond four waves of 256 tracks an
+   * SM. An explicit part disables both; the other parts take defaults (FP64: 128 threads x 2
+   * blocks per SM, 255 registers; mixed: 128 x 4, 128 registers; 32 tracks per warp), as record
+   * capture does. */
   uint32_t flags;
   uint32_t block_threads;
   uint32_t blocks_per_sm;
@@ -220,9 +224,9 @@ typedef struct tkf_fit_options {
    * variance; the mean energy loss given back). The result is the weighted mean of the
    * backward filtered state at the first surface and the seed. It propagates every track twice;
    * no per-measurement state is kept. One lane a track (lanes_per_track 0 or 1), no record
-   * capture; 255 registers, or max_registers 128 / 64 in TKF_FP64 and TKF_MIXED. Default block
-   * shape 128 threads x 2 blocks per SM (x 4 or x 8 when capped at 128 / 64) unless one is
-   * given; TKF_FIT_AUTOTUNE times the block shapes and register caps as for RTS (one lane a
+   * capture; 255 registers, or max_registers 128 / 64 in TKF_FP64 and TKF_MIXED. With a
+   * register cap alone, 128 threads x 2 blocks per SM (x 4 or x 8 when capped at 128 / 64) unless
+   * a block shape is given; TKF_FIT_AUTOTUNE times the block shapes and register caps as for RTS (one lane a
    * track), cached apart from RTS. */
   int smoother;
   /* TKF_SMOOTHER_TWO_FILTER: factor on the last filtered covariance that starts the backward
@@ -244,8 +248,8 @@ typedef struct tkf_fit_options {
  * tuning. If the environment variable TKF_AUTOTUNE_CACHE names a file when the context is
  * created, tuned shapes are read from it and every new one is written back (JSON object:
  * class -> [threads, blocks per SM, tracks per warp, registers]); an unreadable or unwritable
- * file is ignored. Skipped (defaults used) while the stream is capturing and in record-capture
- * mode. */
+ * file is ignored. Skipped (the shape without tuning is used) while the stream is capturing and in
+ * record-capture mode. */
 #define TKF_FIT_AUTOTUNE 1u
 /* Graph replay: the ordering and fit launches of a call are captured into a CUDA graph on the
  * second consecutive call with identical arguments (every pointer, size, option, handle and
@@ -299,15 +303,15 @@ typedef struct tkf_fit_inputs {
  * track, in the measurements' indexing (entry k of track i at column offsets[i] + k; phi in
  * (-pi, pi], angles at entries without a measurement too). They come from the
  * Rauch-Tung-Striebel backward pass over stored filtered and predicted states and transport
- * Jacobians (A_k = C_k|k J_{k+1}^T C_{k+1|k}^-1, Cholesky), FP64, in a second kernel after the
- * fit; the context's workspace then also holds 360 bytes per measurement row. The entry-0 state
+ * Jacobians (A_k = C_k|k J_{k+1}^T C_{k+1|k}^-1, by L D L^T), FP64, in a second kernel after the
+ * fit; the context's workspace then also holds 320 bytes per measurement row. The entry-0 state
  * equals par / cov up to rounding (par / cov come from the forward-evaluated smoother). Rows of
  * a track whose status is fatal, or that has no measurement, are NaN; a predicted covariance that
  * is not positive definite in the backward pass sets TKF_TRACK_SMOOTHER_NOT_SPD (and NaN outputs)
  * as it does in the textbook smoother. Requires TKF_STEP_ADAPTIVE without record capture, the
  * RTS smoother and tkf_fit (not tkf_fit_host or tkf_fit_noalloc; TKF_ERR_UNSUPPORTED otherwise).
- * It runs one lane a track (lanes_per_track is ignored): by default 128 threads x 2 blocks per
- * SM at 255 registers; max_registers 128 / 64 (x 4 / x 8 blocks) where the precision has them;
+ * It runs one lane a track (lanes_per_track is ignored): by default at 255 registers, 128 threads x 2
+ * blocks per SM (one-warp blocks for small batches); max_registers 128 / 64 (x 4 / x 8 blocks) where the precision has them;
  * TKF_FIT_AUTOTUNE times the one-lane shapes and register caps, cached apart from the plain fit.
  * NULL keeps the default path, unchanged and as fast. */
 typedef struct tkf_fit_outputs {
@@ -629,7 +633,8 @@ tkf_status tkf_propose_start(tkf_context ctx, tkf_geometry geo, tkf_field field,
  *     (different streams, or different contexts, without ordering) race and give wrong
  *     results. Serialize them.
  *   - It ignores the flags TKF_FIT_AUTOTUNE and TKF_FIT_GRAPH (both allocate); it launches with
- *     the shape tkf_fit uses without tuning (the explicit one of the options, else the default).
+ *     the shape tkf_fit uses without tuning (the explicit one of the options, else the one by size;
+ *     the two-filter smoother then keeps 255 registers).
  *   - Learned step mode (TKF_STEP_LEARNED) returns TKF_ERR_UNSUPPORTED: it needs a per-track
  *     starting step, for which the static scratch has no room.
  *   - TKF_ERR_DEVICE if the array's address was not found when the context was created.
