@@ -46,6 +46,10 @@ WORKLOAD_MAP = "solenoid_map_100k_muons"
 # in R = P J^T (45 flops fewer per propagated measurement).
 FLOPS = {
     "fp64": (493, 111, 1494, 330),
+    # the FP64 path in a field along z: closed-form steps (34 an attempt; the "fp64" rows are the
+    # stage-by-stage form of any other field)
+    "fp64_axial": (103, 41, 1168, 330),
+    "fp64_axial_two_filter": (103, 41, 1617, 1837),
     # mixed: only the FP64 anchors, the Joseph update and the smoother count
     "mixed": (20, 8, 704, 330),
     "mixed_learned": (20, 8, 704, 330),
@@ -75,22 +79,28 @@ FLOPS_MAP = {
 # launch and are scaled by tracks to a full launch. Keyed by (workload, variant, register cap of
 # the launched kernel); a kernel change voids the entries (profiles/ keeps the commands).
 CAPTURES = {
-    ("barrel", "mixed_learned", 64): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5100920,
-        "rejected": 16960, "shape": "32,32,32,64", "dram_bytes": 8996654080,
-        "fp64_exec": 2383301181, "fp64_model": 2281057572, "fp32_exec": 4787750993},
-    ("barrel", "mixed", 64): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014959,
-        "rejected": 143605, "shape": "32,32,32,64", "dram_bytes": 9000243200,
-        "fp64_exec": 2380095541, "fp64_model": 2277818612, "fp32_exec": 4703923835},
-    ("barrel", "mixed_learned", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5100793,
-        "rejected": 18151, "shape": "128,4,32,128", "dram_bytes": 1410114048,
-        "fp64_exec": 2377319935, "fp64_model": 2281040740, "fp32_exec": 4920394687},
+    ("barrel", "mixed_learned", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5100021,
+        "rejected": 17506, "shape": "128,4,32,128", "dram_bytes": 1495617024,
+        "fp64_exec": 2357505588, "fp64_model": 2281033040, "fp32_exec": 3651469626},
     ("barrel", "mixed", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014959,
-        "rejected": 143605, "shape": "64,8,32,128", "dram_bytes": 1368626432,
-        "fp64_exec": 2374166495, "fp64_model": 2277818612, "fp32_exec": 4828531039},
+        "rejected": 143605, "shape": "128,4,32,128", "dram_bytes": 1458471424,
+        "fp64_exec": 2354693398, "fp64_model": 2277818612, "fp32_exec": 3604152818},
+    ("barrel", "fp64_axial", 255): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014958,
+        "rejected": 143611, "shape": "128,2,32,255", "dram_bytes": 1047469568,
+        "fp64_exec": 4627625879, "fp64_model": 4062418156, "fp32_exec": 207284986},
+    ("barrel", "fp64_axial", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014958,
+        "rejected": 143611, "shape": "128,4,32,128", "dram_bytes": 2143469056,
+        "fp64_exec": 4645413017, "fp64_model": 4062418156, "fp32_exec": 234135716},
+    # the stage-by-stage form, which the FP64 path took on this batch before the closed-form steps
     ("barrel", "fp64", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014958, "rejected": 143611,
                               "shape": "128,4,32,128", "dram_bytes": 2871720960,
                               "fp64_exec": 8183930686, "fp64_model": 6938730754, "fp32_exec": 71595040},
 }
+
+
+def axial_key(variant: str) -> str:
+    """The FLOPS row of a variant in a field along z."""
+    return variant.replace("fp64", "fp64_axial", 1) if variant.startswith("fp64") else variant
 
 
 def fp32_peak_tflops(sm_mhz: float | None):
@@ -944,7 +954,8 @@ def main():
             ckf_mixed = ckf_stage(ctx, fld, w, stream, max(1, args.steps // 2), 1, precision=tkf.MIXED)
     ms, ms_max, clocks = results[head]["ms"], results[head]["ms_max"], results[head]["clocks"]
     for k, v in results.items():
-        counts = (FLOPS_MAP if args.workload == "map" else FLOPS).get(k)  # no count for the two-filter form
+        counts = (FLOPS_MAP.get(k) if args.workload == "map" else
+                  FLOPS.get(axial_key(k)))  # no count for the all-states form
         if counts is None:
             v["flops"] = None
             continue
@@ -984,7 +995,7 @@ def main():
     hv = results[head]
     head_shape = hv["shape"] or [None] * 5
     # the captured kernel: one lane a track (a group shape is another kernel)
-    cap_key = (args.workload, head, head_shape[3]) if (head_shape[4:] or [1])[0] == 1 else None
+    cap_key = (args.workload, axial_key(head) if args.workload == "barrel" else head, head_shape[3]) if (head_shape[4:] or [1])[0] == 1 else None
     cap = CAPTURES.get(cap_key)
     # no FP64 flop count for the two-filter variants: their roofline stays null
     kernel_s = hv["kernel_ms"] * 1e-3
