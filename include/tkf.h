@@ -185,7 +185,7 @@ typedef struct tkf_fit_options {
    * variant capped at that many registers a thread, which keeps part of the per-track state in
    * local memory (at 128 the smoother state in shared memory) and holds more warps per SM. With
    * all four 0 the shape is the tuned one of this launch class when TKF_FIT_AUTOTUNE is set,
-   * else one by the batch's size: four lanes a track up to 80 tracks an SM (RTS without all
+   * else one by the batch's size: four lanes a track up to 56 tracks an SM (RTS without all
    * states), one lane a track and 255 registers above, blocks of one warp while they are fewer
    * than the resident warps, 128 registers for the mixed fit beyond four waves of 256 tracks an
    * SM. An explicit part disables both; the other parts take defaults (FP64: 128 threads x 2

@@ -50,10 +50,11 @@ std::array<int, 5> default_shape(int precision, bool record) {
 // Launch shape without tuning of the FP64 and mixed paths by the batch's size (record capture and explicit
 // options keep the fixed defaults). Sizes are in lanes of the full-register kernels (8 warps an SM: 38,912
 // on 152 SMs); both sides of each line measured on barrel + endcap tracks (uniform field / map), ms:
-// * RTS below 80 tracks an SM (12,160; a wave of four-lane groups is 64 an SM): four lanes a track, the
-//   warps' tracks halved while every SM still gets a warp. FP64 3,000 tracks 0.87 -> 0.55 / 2.96 -> 2.31,
-//   12,500 1.03 -> 0.78 / 3.52 -> 2.60; mixed 3,000 0.36 -> 0.31 / 0.65 -> 0.44, 12,500 0.40 -> 0.40 /
-//   0.63 -> 0.61; at 20,000 one lane wins (mixed 0.46 against 0.55 / 0.65 against 0.88).
+// * RTS up to 56 tracks an SM (8,512; a wave of four-lane groups is 64 an SM): four lanes a track, the warps'
+//   tracks halved while every SM still gets a warp. Groups / one lane: 6,000 tracks mixed 0.255 / 0.308, map
+//   0.43 / 0.49, FP64 0.54 / 0.63, map 1.97 / 2.32; 8,000 mixed 0.284 / 0.314, 0.47 / 0.48, FP64 0.63 / 0.65,
+//   2.44 / 2.23; 9,000 mixed 0.310 / 0.323, 0.501 / 0.503, telescope 0.212 / 0.201, FP64 0.69 / 0.62, 2.46 / 2.34;
+//   12,000 mixed 0.41 / 0.33, 0.59 / 0.50, telescope 0.304 / 0.201, FP64 0.78 / 0.64, 2.60 / 2.22.
 // * mixed: the full register file up to 4 waves, then 128 registers, whose 16 warps an SM hide more than their
 //   spills cost (in step; 255 / 128 registers: 60,000 map 0.83 / 1.00; 100,000 0.95 / 0.97, map 1.24 / 1.25,
 //   two-filter 1.35 / 1.37; 150,000 1.34 / 1.35, 1.69 / 1.65, 1.90 / 1.95; 200,000 1.73 / 1.72, two-filter
@@ -66,7 +67,7 @@ LaunchShape sized_shape(const FitArgs& a, int precision, uint32_t sms) {
   const uint32_t n = a.n_tracks, wave = 32 * kResidentWarpsPerSm * sms;
   const bool two_filter = a.smoother == TKF_SMOOTHER_TWO_FILTER, states = a.states_par != nullptr;
   LaunchShape s;
-  if (!two_filter && !states && n <= 80 * sms) {
+  if (!two_filter && !states && n <= 56 * sms) {
     s.group = 4;
     s.tracks_per_warp = 8;
     while (s.tracks_per_warp > 1 && n <= uint32_t(s.tracks_per_warp / 2) * sms) s.tracks_per_warp /= 2;

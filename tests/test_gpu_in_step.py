@@ -71,9 +71,9 @@ def test_blocks_in_step(ctx, field, smoother, n, shape):
             np.testing.assert_array_equal(getattr(r, k).cpu().numpy(), getattr(out[-1], k).cpu().numpy(), err_msg=k)
 
 
-@pytest.mark.parametrize("per_sm,extra", [(1024, 0), (1024, 1)])
+@pytest.mark.parametrize("per_sm,extra", [(56, 0), (56, 1), (1024, 0), (1024, 1)])
 def test_the_size_without_tuning(ctx, per_sm, extra):
-    """The full register file up to 4 waves, 128 registers beyond."""
+    """Four lanes a track up to 56 tracks an SM; the full register file up to 4 waves, 128 registers beyond."""
     n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
     w = synth.telescope_workload(n, seed=22)
     t = w.tracks
