@@ -1172,7 +1172,7 @@ extern "C" tkf_status tkf_fit_noalloc(tkf_context ctx, tkf_geometry geo, tkf_fie
                                      &shape);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tkf_fit_noalloc: launch shape");
   // the two-filter smoother keeps the full register file (2.49 against 2.47 ms at 200,000 tracks): the spilled state
-  // of its 128-register kernels (0.6 KB a thread) could grow the driver's local-memory pool at launch
+  // of its 128-register kernels (0.6 KB a thread) could grow CUDA's local-memory pool at launch
   if (shape.regs != 255 && o->smoother == TKF_SMOOTHER_TWO_FILTER && !o->max_registers)
     shape = tkf::default_launch_shape(TKF_FP64, false, ctx->sm_count);
   e = tkf::launch_fit(a, field->f, o->precision, ws, shape, static_cast<cudaStream_t>(stream));
