@@ -555,9 +555,13 @@ __device__ int predict(bool go, const CkfArgs& a, const F& fld, const NavTables&
         if (once) return kRetry;
         continue;
       }
-      // bound parameters (FP64 from the anchors) and the transport Jacobian in FP32
-      double sp2, cp2, st2, ct2, inv_st, nrm;
-      bound_direction(T, sp2, cp2, st2, ct2, inv_st, nrm);
+      // bound parameters (FP64 from the anchors) and the transport Jacobian in FP32. The next prediction copies the
+      // direction to FP32, where a last bit can move a copy to its neighbour (6e-8, and chi2 with it): correctly
+      // rounded roots and divisions, not bound_direction's
+      const double inv_norm = 1.0 / sqrt(dot3(T, T));
+      const double tn[3] = {T[0] * inv_norm, T[1] * inv_norm, T[2] * inv_norm};
+      const double st2 = sqrt(tn[0] * tn[0] + tn[1] * tn[1]), inv_st = 1.0 / st2;
+      const double ct2 = tn[2], cp2 = tn[0] * inv_st, sp2 = tn[1] * inv_st;
       const float Tf[3] = {d2f(T[0]), d2f(T[1]), d2f(T[2])};
       const float inv_nT = 1.0f / dotr(s.nf, Tf);
       const float fst = d2f(st2), fct = d2f(ct2), fcp = d2f(cp2), fsp = d2f(sp2), finv_st = d2f(inv_st);
@@ -688,17 +692,20 @@ __device__ int predict(bool go, const CkfArgs& a, const F& fld, const NavTables&
   }
 }
 
+// 1 / det of the residual covariance; correctly rounded in the mixed path, whose filtered state is copied to FP32 (predict)
+template <bool kMixed>
 __device__ __forceinline__ double inverse(double det) {
-  return abs_lt(det, 1e290) && !abs_lt(det, 1e-290) ? rcp_nr(det) : 1.0 / det;
+  return !kMixed && abs_lt(det, 1e290) && !abs_lt(det, 1e-290) ? rcp_nr(det) : 1.0 / det;
 }
 
 // predicted chi2 of a measurement (no update)
+template <bool kMixed>
 __device__ __forceinline__ bool meas_chi2(const double pp[5], const double Cp[15], double m0, double m1, double V00,
                                           double V01, double V11, double& chi2) {
   const double S00 = Cp[S(0, 0)] + V00, S01 = Cp[S(0, 1)] + V01, S11 = Cp[S(1, 1)] + V11;
   const double det = S00 * S11 - S01 * S01;
   if (!(positive(S00) && positive(det))) return false;
-  const double idet = inverse(det);
+  const double idet = inverse<kMixed>(det);
   const double Si00 = S11 * idet, Si01 = -S01 * idet, Si11 = S00 * idet;
   const double r0 = m0 - pp[0], r1 = m1 - pp[1];
   chi2 = r0 * (Si00 * r0 + Si01 * r1) + r1 * (Si01 * r0 + Si11 * r1);
@@ -706,10 +713,11 @@ __device__ __forceinline__ bool meas_chi2(const double pp[5], const double Cp[15
 }
 
 // gain-matrix update, Joseph form (as in the fit)
+template <bool kMixed>
 __device__ void update(double p[5], double C[15], double m0, double m1, double V00, double V01, double V11,
                        double& chi2) {
   const double S00 = C[S(0, 0)] + V00, S01 = C[S(0, 1)] + V01, S11 = C[S(1, 1)] + V11;
-  const double idet = inverse(S00 * S11 - S01 * S01);
+  const double idet = inverse<kMixed>(S00 * S11 - S01 * S01);
   const double Si00 = S11 * idet, Si01 = -S01 * idet, Si11 = S00 * idet;
   const double r0 = m0 - p[0], r1 = m1 - p[1];
   chi2 = r0 * (Si00 * r0 + Si01 * r1) + r1 * (Si01 * r0 + Si11 * r1);
@@ -1097,6 +1105,7 @@ __global__ void __launch_bounds__(kCkfBlock) ckf_predict_kernel(const CkfArgs a,
 }
 
 // Phase 2: the gate over the predicted module's measurements and the children of branch bi.
+template <bool kMixed>
 __global__ void __launch_bounds__(kCkfBlock, 4) ckf_gate_kernel(const CkfArgs a, CkfWork w) {
   const uint32_t B = a.beam;
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1162,7 +1171,7 @@ __global__ void __launch_bounds__(kCkfBlock, 4) ckf_gate_kernel(const CkfArgs a,
       const uint32_t mi = chunk + uint32_t(__ffsll((long long)pass) - 1);
       pass &= pass - 1ull;
       double c2;
-      if (!meas_chi2(pp, Cp, a.loc0[mi], a.loc1[mi], a.v00[mi], a.v01[mi], a.v11[mi], c2)) continue;
+      if (!meas_chi2<kMixed>(pp, Cp, a.loc0[mi], a.loc1[mi], a.v00[mi], a.v01[mi], a.v11[mi], c2)) continue;
       if (!(c2 < a.chi2_max)) continue;
       int pos = nk;
       while (pos > 0 && (c2 < kc2[pos - 1] || (c2 == kc2[pos - 1] && mi < km[pos - 1]))) --pos;
@@ -1182,11 +1191,11 @@ __global__ void __launch_bounds__(kCkfBlock, 4) ckf_gate_kernel(const CkfArgs a,
     for (int j = 0; j < 15; ++j) C[j] = Cp[j];
     const uint32_t mi = km[q];
     double c2;
-    update(p, C, a.loc0[mi], a.loc1[mi], a.v00[mi], a.v01[mi], a.v11[mi], c2);
+    update<kMixed>(p, C, a.loc0[mi], a.loc1[mi], a.v00[mi], a.v01[mi], a.v11[mi], c2);
     // filtered direction: the predicted one turned by the update's angle increments
     double sd, cd, se, ce;
-    small_sincos(p[2], sd, cd);
-    small_sincos(p[3], se, ce);
+    small_sincos<!kMixed>(p[2], sd, cd);
+    small_sincos<!kMixed>(p[3], se, ce);
     CkfBranch& ch = kids[q];
     const double dir[4] = {pdir[0] * cd + pdir[1] * sd, pdir[1] * cd - pdir[0] * sd, pdir[2] * ce + pdir[3] * se,
                            pdir[3] * ce - pdir[2] * se};
@@ -1351,11 +1360,12 @@ cudaError_t launch_ckf(const CkfArgs& a_in, const F& fld, cudaStream_t stream) {
   if ((e = cudaMemsetAsync(w.count, 0, 2 * sizeof(uint32_t), stream)) != cudaSuccess) return e;
   ckf_nav_kernel<<<1, kCkfBlock, 0, stream>>>(a, nav);
   ckf_init_kernel<<<gs, kCkfBlock, 0, stream>>>(a, w);
+  auto* gate = a.mixed ? ckf_gate_kernel<true> : ckf_gate_kernel<false>;
   // every step adds an entry to each surviving branch: at most max_entries + 2 steps
   const uint32_t n_steps = ckf_steps(a.max_entries);
   for (uint32_t step = 0; step < n_steps; ++step) {
     predict<<<gp, kCkfBlock, 0, stream>>>(a, fld, w);
-    ckf_gate_kernel<<<gb, kCkfBlock, 0, stream>>>(a, w);
+    gate<<<gb, kCkfBlock, 0, stream>>>(a, w);
     if ((e = cudaMemsetAsync(w.count, 0, 2 * sizeof(uint32_t), stream)) != cudaSuccess) return e;
     ckf_beam_kernel<<<gs, kCkfBlock, 0, stream>>>(a, w, step, step + 1 == n_steps ? 1u : 0u);
   }

@@ -972,9 +972,10 @@ __device__ __forceinline__ uint32_t material_mixed(const Surf& s, const Material
 }
 
 // sin and cos of a small angle: Taylor polynomials through x^9 / x^8 (truncation below
-// 1e-19 for |x| < 1/16), else the library sincos.
+// 1e-19 for |x| < 1/16), else the library sincos. kShort: fewer terms below 1/512, whose last bits round differently.
+template <bool kShort = true>
 __device__ __forceinline__ void small_sincos(double x, double& s, double& c) {
-  if (abs_lt(x, 1.0 / 512)) {  // through x^5 / x^4: truncation below 2^-65
+  if (kShort && abs_lt(x, 1.0 / 512)) {  // through x^5 / x^4: truncation below 2^-65
     const double x2 = __dmul_rn(x, x);
     s = fma(__dmul_rn(x, x2), fma(x2, 1.0 / 120, -1.0 / 6), x);
     c = fma(x2, fma(x2, 1.0 / 24, -0.5), 1.0);
