@@ -1205,8 +1205,9 @@ __device__ __forceinline__ void transport_cov(const R J[5][5], R Cw[15], uint32_
 // measurement of entry m: sets the gain K, the inverse residual covariance Si and the residual r,
 // updates p and C and adds r^T Si r to chi2. Returns TKF_TRACK_UPDATE_NOT_SPD (state untouched)
 // when the residual covariance is not positive definite.
-// FP64 covariances take the determinant's reciprocal by rcp_nr and test signs on the integer pipe.
-template <int kG, class U>
+// FP64 covariances test signs on the integer pipe; the FP64 fit takes the determinant's reciprocal by rcp_nr, the
+// mixed fit divides: the next propagation copies the filtered state to FP32, where a last bit can move a copy to its neighbour.
+template <int kG, bool kMixed, class U>
 __device__ __forceinline__ uint32_t kalman_update(const FitArgs& a, uint32_t m, double p[5], U C[15], U K[5][2],
                                                   U& Si00, U& Si01, U& Si11, U& r0, U& r1, double& chi2,
                                                   uint32_t gl, uint32_t gmask) {
@@ -1216,7 +1217,7 @@ __device__ __forceinline__ uint32_t kalman_update(const FitArgs& a, uint32_t m, 
   const U det = S00 * S11 - S01 * S01;
   if (!(positive(S00) && positive(det))) return TKF_TRACK_UPDATE_NOT_SPD;
   U idet;
-  if constexpr (sizeof(U) == 8)
+  if constexpr (!kMixed)
     idet = abs_lt(det, 1e290) && !abs_lt(det, 1e-290) ? rcp_nr(det) : 1.0 / det;
   else
     idet = U(1) / det;
@@ -1909,7 +1910,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
     for (int j = 0; j < 5; ++j) K[j][0] = K[j][1] = U(0);
     if (measured) {
       // the track's chi2 is the forward filter's; the backward filter's goes to chi2_bwd
-      status |= kalman_update<kG>(a, m, p, C, K, Si00, Si01, Si11, r0, r1, bwd ? chi2_bwd : chi2, gl, gmask);
+      status |= kalman_update<kG, kMixed>(a, m, p, C, K, Si00, Si01, Si11, r0, r1, bwd ? chi2_bwd : chi2, gl, gmask);
       if (status & kFatal) TKF_LEAVE_ENTRY;
     }  // measured
     if (!bwd && k == 0) {
