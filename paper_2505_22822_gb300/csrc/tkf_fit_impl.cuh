@@ -211,10 +211,12 @@ __device__ __forceinline__ R dotr(const R a[3], const R b[3]) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
+// One order of roundings in FP32: left to the compiler, the kernel at 255 registers in step fused the other product
+// of each difference in a tilted uniform field (covariances 4e-5 off the other kernels').
 __device__ __forceinline__ void cross(const float a[3], const float b[3], float o[3]) {
-  o[0] = a[1] * b[2] - a[2] * b[1];
-  o[1] = a[2] * b[0] - a[0] * b[2];
-  o[2] = a[0] * b[1] - a[1] * b[0];
+  o[0] = fmaf(a[1], b[2], -__fmul_rn(a[2], b[1]));
+  o[1] = fmaf(a[2], b[0], -__fmul_rn(a[0], b[2]));
+  o[2] = fmaf(a[0], b[1], -__fmul_rn(a[1], b[0]));
 }
 
 __device__ __forceinline__ void cross(const double a[3], const double b[3], double o[3]) {
