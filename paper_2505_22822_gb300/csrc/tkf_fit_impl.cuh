@@ -89,7 +89,7 @@ __device__ __forceinline__ void reload_uvf(const double* __restrict__ g, uint32_
 }
 
 __device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+  return fma(a[2], b[2], mul_add(a[0], b[0], a[1], b[1]));
 }
 
 // ------------------------------------------------------------------ field policies
@@ -184,7 +184,7 @@ struct FieldGrid {
   }
   // the same interpolation in FP32 (mixed precision)
   __device__ __forceinline__ void atf(const float* x, float B[3], bool& oof) const {
-    const float r = sqrtf(x[0] * x[0] + x[1] * x[1]);
+    const float r = sqrtf(mul_add(x[0], x[0], x[1], x[1]));
     const float fr = (r - r0f) * inv_drf;
     const float fz = (x[2] - z0f) * inv_dzf;
     if (!(fr >= 0.0f && fr <= rmaxf && fz >= 0.0f && fz <= zmaxf)) {
@@ -197,8 +197,9 @@ struct FieldGrid {
     const float a = fr - ir, b = fz - iz;
     const float2* g = grid + size_t(iz) * nr + ir;
     const float2 g00 = __ldg(g), g01 = __ldg(g + 1), g10 = __ldg(g + nr), g11 = __ldg(g + nr + 1);
-    const float br = (1.0f - b) * ((1.0f - a) * g00.x + a * g01.x) + b * ((1.0f - a) * g10.x + a * g11.x);
-    const float bz = (1.0f - b) * ((1.0f - a) * g00.y + a * g01.y) + b * ((1.0f - a) * g10.y + a * g11.y);
+    const float a1 = 1.0f - a, b1 = 1.0f - b;
+    const float br = mul_add(b1, mul_add(a1, g00.x, a, g01.x), b, mul_add(a1, g10.x, a, g11.x));
+    const float bz = mul_add(b1, mul_add(a1, g00.y, a, g01.y), b, mul_add(a1, g10.y, a, g11.y));
     const float q = r > 0.0f ? br / r : 0.0f;
     B[0] = q * x[0];
     B[1] = q * x[1];
@@ -208,15 +209,16 @@ struct FieldGrid {
 
 template <class R>
 __device__ __forceinline__ R dotr(const R a[3], const R b[3]) {
-  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+  return fma(a[2], b[2], mul_add(a[0], b[0], a[1], b[1]));
 }
 
-// One order of roundings in FP32: left to the compiler, the kernel at 255 registers in step fused the other product
-// of each difference in a tilted uniform field (covariances 4e-5 off the other kernels').
+// The mixed path's sums of two products are written as mul_add and mul_sub. Left to the compiler, the kernel at 255
+// registers in step fused the other product of each difference here, in a tilted uniform field: covariances 4e-5 off the
+// other kernels'. The order of each is the one that all the other kernels had.
 __device__ __forceinline__ void cross(const float a[3], const float b[3], float o[3]) {
-  o[0] = fmaf(a[1], b[2], -__fmul_rn(a[2], b[1]));
-  o[1] = fmaf(a[2], b[0], -__fmul_rn(a[0], b[2]));
-  o[2] = fmaf(a[0], b[1], -__fmul_rn(a[1], b[0]));
+  o[0] = mul_sub(a[1], b[2], a[2], b[1]);
+  o[1] = mul_sub(a[2], b[0], a[0], b[2]);
+  o[2] = mul_sub(a[0], b[1], a[1], b[0]);
 }
 
 __device__ __forceinline__ void cross(const double a[3], const double b[3], double o[3]) {
@@ -717,7 +719,7 @@ __device__ __forceinline__ float step_factor_f(float q) {
 
 __device__ __forceinline__ float parabolic_path_f(float d, float a, float b) {
   float s = d / a;
-  const float disc = a * a + 2.0f * b * d;
+  const float disc = mul_add(a, a, 2.0f * b, d);
   if (disc >= 0.0f) {
     const float q = 2.0f * d / (a + copysignf(sqrtf(disc), a));
     if (isfinite(q)) s = q;
@@ -744,7 +746,7 @@ __device__ uint32_t propagate_mixed(const F& fld, const OptionsDev& o, const Sur
   const float lk = d2f(lam * kKappa);
   const float tol = o.tol_f, h_min = o.h_min_f, h_max = o.h_max_f, surf_tol = o.surf_tol_f;
   for (;;) {
-    const double dist = s.n[0] * (s.c[0] - r[0]) + s.n[1] * (s.c[1] - r[1]) + s.n[2] * (s.c[2] - r[2]);
+    const double dist = fma(s.n[2], s.c[2] - r[2], mul_add(s.n[0], s.c[0] - r[0], s.n[1], s.c[1] - r[1]));
     const float Tf[3] = {d2f(T[0]), d2f(T[1]), d2f(T[2])};
     float rf[3] = {0.0f, 0.0f, 0.0f};
     if (!F::kUniform || kMode == kRecord)
@@ -768,7 +770,7 @@ __device__ uint32_t propagate_mixed(const F& fld, const OptionsDev& o, const Sur
           for (int i = 0; i < kXY; ++i) q[i] += kCols == 1 ? qcol * e[i] : e[i];
         }
         for (int i = 0; i < kXY; ++i) {
-          dr[c][i] += sp * dT[c][i] + sp2 * q[i];
+          dr[c][i] += mul_add(sp, dT[c][i], sp2, q[i]);
           dT[c][i] += sp * q[i];
         }
         if (F::kAlongZ) dr[c][2] = __fadd_rn(dr[c][2], __fmul_rn(sp, dT[c][2]));
@@ -860,7 +862,7 @@ __device__ uint32_t propagate_mixed(const F& fld, const OptionsDev& o, const Sur
         for (int i = 0; i < kXY; ++i) q4[i] += kCols == 1 ? qcol * e[i] : e[i];
       }
       for (int i = 0; i < kXY; ++i) {
-        dr[c][i] += h * dT[c][i] + h * h6 * (q1[i] + q2[i] + q3[i]);
+        dr[c][i] += mul_add(h, dT[c][i], h * h6, q1[i] + q2[i] + q3[i]);
         dT[c][i] += h6 * (q1[i] + 2.0f * q2[i] + 2.0f * q3[i] + q4[i]);
       }
       if (F::kAlongZ) dr[c][2] = __fadd_rn(dr[c][2], __fmul_rn(h, dT[c][2]));
@@ -965,7 +967,7 @@ __device__ __forceinline__ uint32_t material_mixed(const Surf& s, const Material
     bracket = 0.5f * logf(m.two_me_over_i2_f * bg2 * wmax) - beta2;
   const float dE = m.dedx_scale_f * inv_beta2 * bracket * x;
   if (!kGain && !(dE < E - mass)) return TKF_TRACK_PARTICLE_STOPPED;
-  const float delta = kGain ? -(2.0f * E * dE + dE * dE) * l2 : (2.0f * E * dE - dE * dE) * l2;
+  const float delta = kGain ? -mul_add(2.0f * E, dE, dE, dE) * l2 : mul_sub(2.0f * E, dE, dE, dE) * l2;
   const float g = (kGain ? fabsf(delta) < 0.01f : delta < 0.01f)
                       ? delta * (0.5f + delta * (0.375f + delta * (0.3125f + delta * (0.2734375f + delta * 0.24609375f))))
                       : rsqrtf(1.0f - delta) - 1.0f;
@@ -1117,8 +1119,8 @@ __device__ __forceinline__ void jac_column(const R n[3], const R u[3], const R v
   }
   out[0] = dotr(u, x);
   out[1] = dotr(v, x);
-  out[2] = (-sp2 * t[0] + cp2 * t[1]) * inv_st;
-  out[3] = ct2 * cp2 * t[0] + ct2 * sp2 * t[1] - st2 * t[2];
+  out[2] = mul_sub(cp2, t[1], sp2, t[0]) * inv_st;
+  out[3] = fma(-st2, t[2], mul_add(ct2 * cp2, t[0], ct2 * sp2, t[1]));
 }
 
 // a0 b0 + a1 b1, rounded as the full five-term sum with zeros elsewhere
@@ -1216,7 +1218,7 @@ __device__ __forceinline__ uint32_t kalman_update(const FitArgs& a, uint32_t m, 
   const double m0 = a.loc0[m], m1 = a.loc1[m];
   const U V00 = cov_from_d<U>(a.v00[m]), V01 = cov_from_d<U>(a.v01[m]), V11 = cov_from_d<U>(a.v11[m]);
   const U S00 = C[S(0, 0)] + V00, S01 = C[S(0, 1)] + V01, S11 = C[S(1, 1)] + V11;
-  const U det = S00 * S11 - S01 * S01;
+  const U det = mul_sub(S00, S11, S01, S01);
   if (!(positive(S00) && positive(det))) return TKF_TRACK_UPDATE_NOT_SPD;
   U idet;
   if constexpr (!kMixed)
@@ -1228,12 +1230,12 @@ __device__ __forceinline__ uint32_t kalman_update(const FitArgs& a, uint32_t m, 
   Si11 = S00 * idet;
   r0 = cov_from_d<U>(m0 - p[0]);
   r1 = cov_from_d<U>(m1 - p[1]);
-  chi2 += cov_to_d(r0 * (Si00 * r0 + Si01 * r1) + r1 * (Si01 * r0 + Si11 * r1));
+  chi2 += cov_to_d(mul_add(r0, mul_add(Si00, r0, Si01, r1), r1, mul_add(Si01, r0, Si11, r1)));
 #pragma unroll
   for (int j = 0; j < 5; ++j) {
     const U U0 = C[S(j, 0)], U1 = C[S(j, 1)];
-    K[j][0] = U0 * Si00 + U1 * Si01;
-    K[j][1] = U0 * Si01 + U1 * Si11;
+    K[j][0] = mul_add(U0, Si00, U1, Si01);
+    K[j][1] = mul_add(U0, Si01, U1, Si11);
   }
 #pragma unroll
   for (int j = 0; j < 5; ++j) p[j] = add2d(p[j], K[j][0], r0, K[j][1], r1);
@@ -1297,10 +1299,10 @@ __device__ __forceinline__ bool turn_direction(const double p[5], double sp2, do
     double sd, cd1, se, ce1;
     small_sincos_m1(p[2], sd, cd1);
     small_sincos_m1(p[3], se, ce1);
-    sph = sp2 + (sp2 * cd1 + cp2 * sd);
-    cph = cp2 + (cp2 * cd1 - sp2 * sd);
-    sth = st2 + (st2 * ce1 + ct2 * se);
-    cth = ct2 + (ct2 * ce1 - st2 * se);
+    sph = sp2 + mul_add(cp2, sd, sp2, cd1);
+    cph = cp2 + mul_sub(cp2, cd1, sp2, sd);
+    sth = st2 + mul_add(ct2, se, st2, ce1);
+    cth = ct2 + mul_sub(ct2, ce1, st2, se);
   }
   return positive(sth);
 }
@@ -1452,7 +1454,7 @@ __device__ __forceinline__ uint32_t combine_with_seed(const FitArgs& a, uint32_t
     for (int c = r; c < 5; ++c) {
       U acc = A[r][c];
 #pragma unroll
-      for (int q = 0; q < 5; ++q) acc += B[r][q] * K[c][q] - A[r][q] * K[c][q];
+      for (int q = 0; q < 5; ++q) acc += mul_sub(B[r][q], K[c][q], A[r][q], K[c][q]);
       st.E(S(r, c)) = acc;
     }
   return 0;
@@ -1777,7 +1779,7 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       const double t2 = dot3(T, T), e2 = t2 - 1.0;
       const double inv_norm = abs_lt(e2, 1e-4) ? 1.0 - e2 * (0.5 - 0.375 * e2) : 1.0 / sqrt(t2);
       const double tn[3] = {T[0] * inv_norm, T[1] * inv_norm, T[2] * inv_norm};
-      const double v = tn[0] * tn[0] + tn[1] * tn[1];
+      const double v = mul_add(tn[0], tn[0], tn[1], tn[1]);
       double inv_st;
       if (!abs_le(v, 1e-12)) {  // v >= 0
         const float yf = sqrtf(d2f(v));
@@ -1957,8 +1959,8 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       U W[5][2];
 #pragma unroll
       for (int j = 0; j < 5; ++j) {
-        W[j][0] = st.P(j, 0) * Si00 + st.P(j, 1) * Si01;
-        W[j][1] = st.P(j, 0) * Si01 + st.P(j, 1) * Si11;
+        W[j][0] = mul_add(st.P(j, 0), Si00, st.P(j, 1), Si01);
+        W[j][1] = mul_add(st.P(j, 0), Si01, st.P(j, 1), Si11);
         st.dl(j) = add2d(st.dl(j), W[j][0], r0, W[j][1], r1);
       }
 #pragma unroll
@@ -1974,8 +1976,8 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
       }
       } else {
         // rows gl and 4; columns 0 and 1 of R from every row's lane
-        const U Wg0 = Pg[0] * Si00 + Pg[1] * Si01, Wg1 = Pg[0] * Si01 + Pg[1] * Si11;
-        const U W40 = P4[0] * Si00 + P4[1] * Si01, W41 = P4[0] * Si01 + P4[1] * Si11;
+        const U Wg0 = mul_add(Pg[0], Si00, Pg[1], Si01), Wg1 = mul_add(Pg[0], Si01, Pg[1], Si11);
+        const U W40 = mul_add(P4[0], Si00, P4[1], Si01), W41 = mul_add(P4[0], Si01, P4[1], Si11);
         dlg = add2d(dlg, Wg0, r0, Wg1, r1);
         dl4 = add2d(dl4, W40, r0, W41, r1);
         U R0c[5], R1c[5];

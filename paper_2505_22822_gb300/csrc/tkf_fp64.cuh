@@ -71,6 +71,19 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   return fma(__dmul_rn(y, e), fma(e, 0.375, 0.5), y);
 }
 
+// a b + c d and a b - c d with the first product fused and the second rounded. Which of two products a compiler fuses
+// depends on what surrounds the sum: left to it, kernels of the same source round differently.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <class R>
+__device__ __forceinline__ R mul_add(R a, R b, R c, R d) {
+  return fma(a, b, mul_rn(c, d));
+}
+template <class R>
+__device__ __forceinline__ R mul_sub(R a, R b, R c, R d) {
+  return fma(a, b, -mul_rn(c, d));
+}
+
 // a . b with a fixed order of roundings
 __device__ __forceinline__ double dot3f(const double a[3], const double b[3]) {
   return fma(a[2], b[2], fma(a[1], b[1], __dmul_rn(a[0], b[0])));
