@@ -1497,11 +1497,28 @@ __device__ __forceinline__ void store_predicted(const FitArgs& a, uint32_t m, co
   }
 }
 
-// kStep: every lane of the block calls this together, lanes that are not live only keep step
+// In step: the warps of a block meet before each entry, so that they run the same code at the same time. The meeting
+// orders no data: a warp posts the entries it has passed (`now`) and waits for the others of its block, but for no more
+// than kMeetPolls polls (about 0.1 ms, a few entries' time) and not for one that is two entries behind. A track that curls
+// for thousands of steps then holds its own warp alone: eight such tracks, each at another entry, in the eight
+// warps of a block took 64.5 ms with a block barrier and take 8.2, as long as one of them. Where no track lags, the
+// times are the barrier's (600,000 learned 4.93 / 4.92, map 100,000 1.22 / 1.22, two-filter 200,000 2.45 / 2.45 ms).
+constexpr int kMeetPolls = 4096;
+__device__ __forceinline__ void keep_step(volatile uint32_t* passed, uint32_t now) {
+  const uint32_t lane = threadIdx.x & 31u, warps = blockDim.x >> 5;
+  __syncwarp();
+  if (lane == 0) passed[threadIdx.x >> 5] = now;
+  for (int it = 0; it < kMeetPolls; ++it) {
+    const uint32_t v = lane < warps ? passed[lane] : now;
+    if (__all_sync(0xffffffffu, v >= now || v + 1u < now || lane == (threadIdx.x >> 5))) break;
+  }
+}
+
+// kStep: every lane of the block calls this together, lanes that are not live only keep step (`passed`: a word a warp)
 template <int kPrec, int kMode, int kG, int kPlace, int kSmooth, bool kRoll, bool kStep, class F>
 __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
                           SmootherStore<kPlace, typename CovType<kPrec>::type> st, uint32_t gl, uint32_t gmask,
-                          bool live, int n_max) {
+                          bool live, int n_max, volatile uint32_t* passed) {
   constexpr bool kMixed = kPrec != 0;
   static_assert(kG == 1 || kMode != kRecord, "record capture runs one lane per track");
   static_assert(kSmooth == 0 || (kG == 1 && kMode != kRecord), "the two-filter smoother runs one lane a track");
@@ -1585,11 +1602,11 @@ __device__ void fit_track(const FitArgs& a, const F& fld, uint32_t i,
     if (!kStep && (status & kFatal)) break;
     if (!(status & kFatal)) reverse_for_backward(p, C, sph, cph, cth, U(a.backward_inflation));
   }
-  // in step, every lane of the block passes n_max barriers: its own entries first, then none
+  // in step, every lane of the block passes n_max meetings: its own entries first, then none
   for (int ent = 0; kStep ? ent < n_max : (ent < N && !(status & kFatal)); ++ent) {
-    if constexpr (kStep) __syncthreads();
+    if constexpr (kStep) keep_step(passed, uint32_t(pass * n_max + ent + 1));
     if (!kStep || (ent < N && !(status & kFatal))) do {
-// a fatal status ends the track: out of the loop, or past the rest of the entry to the next barrier
+// a fatal status ends the track: out of the loop, or past the rest of the entry to the next meeting
 #define TKF_LEAVE_ENTRY      \
   if constexpr (kStep) break; \
   else goto entries_done
@@ -2089,10 +2106,10 @@ __host__ __device__ constexpr int reg_min_blocks(int regs) { return regs >= 255 
 // warps would take the L1 capacity those spills need: launch +6 %).
 __host__ __device__ constexpr int reg_state_place(int regs) { return regs == 128 ? 2 : 0; }
 
-// Fits whose block passes its entries in step, with one barrier an entry: the mixed fit at one lane a track. Its
+// Fits whose block passes its entries in step, with one meeting an entry: the mixed fit at one lane a track. Its
 // entry is a long stretch of straight code, and waiting for instructions was its first stall (in the field map 8.8
 // warps an issue): warps that run the same stretch together share each fetch. The block takes tpw tracks a warp at
-// once and every lane passes as many barriers as its longest track has entries; the ordering by length keeps
+// once and every lane passes as many meetings as its longest track has entries; the ordering by length keeps
 // the idle ones few. 128-thread blocks, ms without / with, at 128 and at 255 registers:
 //   uniform field 200,000 tracks 1.80 / 1.72, 1.84 / 1.73, learned 600,000 5.20 / 4.98, 5.49 / 4.99;
 //   field map 300,000 3.50 / 3.12, 3.93 / 3.21, 100,000 1.34 / 1.25, 1.49 / 1.24;
@@ -2123,11 +2140,12 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
   const uint32_t g = lane / kG, gl = lane % kG;
   const uint32_t gmask = kG == 1 ? 0xffffffffu : ((1u << kG) - 1u) << (g * kG);
   if constexpr (in_step(kPrec, kMode, kRegs, kG)) {
-    __shared__ uint32_t next;
+    __shared__ uint32_t next, passed[reg_block_threads(kRegs) / 32];
     __shared__ int longest;
     const uint32_t first = (threadIdx.x >> 5) * tpw + g;  // this lane's track of the block's share
     for (;;) {
       __syncthreads();
+      if (threadIdx.x < blockDim.x / 32) passed[threadIdx.x] = 0;
       if (threadIdx.x == 0) {
         next = atomicAdd(counter, tpw * (blockDim.x >> 5));
         longest = 0;
@@ -2141,7 +2159,7 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
       const uint32_t b0 = a.offsets[i], b1 = a.offsets[i + 1];
       if (b1 >= b0 && b1 <= a.n_meas) atomicMax(&longest, int(b1 - b0));
       __syncthreads();
-      fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll, true>(a, fld, i, st, gl, gmask, live, longest);
+      fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll, true>(a, fld, i, st, gl, gmask, live, longest, passed);
     }
   } else {
     for (;;) {
@@ -2151,7 +2169,7 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
       if (base >= a.n_tracks) break;
       const uint32_t j = base + g;
       if (g < tpw && j < a.n_tracks)
-        fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll, false>(a, fld, perm[j], st, gl, gmask, true, 0);
+        fit_track<kPrec, kMode, kG, kPlace, kSmooth, kRoll, false>(a, fld, perm[j], st, gl, gmask, true, 0, nullptr);
     }
   }
 }
