@@ -2507,7 +2507,18 @@ cudaError_t launch_persistent(const FitArgs& a, const F& fld, const uint32_t* pe
   // no more blocks than shares of tracks: the block scheduler then spreads a small batch over the SMs, where the
   // first blocks would take it all (mixed, 128 x 2 at 255 registers: 20,000 tracks 0.44 -> 0.37 ms, in the field map
   // 0.65 -> 0.53, two-filter 10,000 0.64 -> 0.51)
-  const uint32_t share = uint32_t(shape.tracks_per_warp) * uint32_t(shape.threads / 32);
+  const uint32_t warps = uint32_t(shape.threads / 32);
+  if constexpr (in_step(kPrec, kMode, kRegs, kG)) {
+    // a block in step takes the shares of its warps at once: none so large that an SM is left without a block
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const uint32_t one_each = warps * uint32_t(std::max(1, std::min(sms, shape.blocks)));
+    shape.tracks_per_warp = int(std::min<uint64_t>(uint64_t(shape.tracks_per_warp),
+                                                   (uint64_t(a.n_tracks) + one_each - 1) / one_each));
+  }
+  const uint32_t share = uint32_t(shape.tracks_per_warp) * warps;
   shape.blocks = std::min(shape.blocks, std::max(1, int((uint64_t(a.n_tracks) + share - 1) / share)));
   fit_persistent_kernel<kPrec, kMode, kRegs, kG, kSmooth>
       <<<shape.blocks, shape.threads, smem, stream>>>(a, fld, perm, counter, uint32_t(shape.tracks_per_warp));

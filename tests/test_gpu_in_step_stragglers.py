@@ -57,3 +57,31 @@ def test_warps_wait_a_while(smoother, threads, registers):
     for k in ("status", "steps"):
         np.testing.assert_array_equal(getattr(got, k).cpu().numpy(), getattr(want, k).cpu().numpy(), err_msg=k)
     assert together < 1.5 * alone, (together, alone)
+
+
+def test_a_small_batch_reaches_every_sm():
+    """A block takes the shares of its warps at once; 600 tracks in blocks of four warps are spread over the SMs as if
+    a warp asked for one track, not handed to five blocks."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ctx = tkf.Context(0)
+    w = synth.solenoid_muon_workload(600, seed=35)
+    t = w.tracks
+    b = tkf.Batch.from_arrays(t.offsets, t.meas, t.sid, t.seed_par, t.seed_cov).to("cuda:0")
+    geo, fld = tkf.Geometry.from_table(ctx, w.geometry.table), tkf.Field.from_desc(ctx, w.field)
+
+    def run(**kw):
+        o = tkf.Options(precision=tkf.MIXED, mass=w.mass, block_threads=128, blocks_per_sm=4, max_registers=128, **kw)
+        times = []
+        for _ in range(21):
+            begin, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            begin.record()
+            tkf.fit(ctx, geo, fld, b, o)
+            end.record()
+            torch.cuda.synchronize()
+            times.append(begin.elapsed_time(end))
+        return sorted(times)[10]
+
+    run()
+    spread, default = run(tracks_per_warp=1), run()
+    assert default < 1.12 * spread, (default, spread)
