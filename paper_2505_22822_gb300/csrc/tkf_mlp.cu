@@ -11,8 +11,8 @@
 //     FP32; each CTA writes its partial gradient;
 //   then the partials summed in CTA order (no atomics: deterministic) and the Adam step.
 // mlp_train_steps_kernel runs up to 256 steps in one cooperative launch; mlp_train_tc_kernel and
-// mlp_reduce_adam_kernel are one step in two launches (the gradient alone, and devices whose SMs
-// cannot hold a batch's CTAs at once).
+// mlp_reduce_adam_kernel are one step in two launches (the gradient alone, and devices that cannot hold a
+// batch's CTAs at once).
 // Around training: seeded initialisation, calibration of the output bias (a quantile of the
 // training residuals, by a radix select on the device) and rounding to the BF16 weights the
 // fit's inference uses.
@@ -794,23 +794,59 @@ TrainScratch carve_train(void* base, uint32_t batch) {
 constexpr size_t kTrainSmemBytes = sizeof(TrainSmem) + 1024;  // + alignment slack
 static_assert(kTrainSmemBytes <= 227 * 1024, "shared memory");
 
-// Whether a batch's CTAs can run at the same time on this device (one an SM), as the steps kernel
-// needs; the largest batch has 64. A device partition with fewer SMs trains step by step.
-bool train_together(unsigned n_cta) {
-  int dev = 0, sms = 0, coop = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
-      cudaFuncSetAttribute(mlp_train_steps_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(kTrainSmemBytes)) != cudaSuccess ||
-      cudaFuncSetAttribute(mlp_train_steps_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(kTrainSmemBytes)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_steps_kernel<false>, kTrainThreads,
-                                                    kTrainSmemBytes) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+// How a batch's CTAs can run at the same time on this device, as the steps kernel needs (one an SM; the largest batch
+// has 64): as one cluster (2, 4 or 8 CTAs: batches of 129 to 256, 385 to 512 and 897 to 1,024; its barrier takes a fifth of
+// the counter's time) where the device says that it can place one, else as a cooperative launch, else not at all.
+// A device partition without room for them trains step by step.
+enum class Together { kNo, kCooperative, kCluster };
+
+struct StepsConfig {
+  cudaLaunchAttribute attr{};
+  cudaLaunchConfig_t cfg{};
+  StepsConfig(unsigned n_cta, Together how, cudaStream_t stream) {
+    if (how == Together::kCluster) {
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = n_cta;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    } else {
+      attr.id = cudaLaunchAttributeCooperative;
+      attr.val.cooperative = 1;
+    }
+    cfg.gridDim = dim3(n_cta);
+    cfg.blockDim = dim3(kTrainThreads);
+    cfg.dynamicSmemBytes = kTrainSmemBytes;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
   }
-  return coop && n_cta <= unsigned(sms) * unsigned(per_sm);
+  StepsConfig(const StepsConfig&) = delete;  // cfg points to attr
+};
+
+Together train_together(unsigned n_cta) {
+  int dev = 0, sms = 0, coop = 0, per_sm = 0, clusters = 0;
+  const StepsConfig cluster(n_cta, Together::kCluster, nullptr);
+  if (cudaGetDevice(&dev) == cudaSuccess && (n_cta == 2 || n_cta == 4 || n_cta == 8) &&
+      cudaFuncSetAttribute(mlp_train_steps_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(kTrainSmemBytes)) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&clusters, mlp_train_steps_kernel<true>, &cluster.cfg) == cudaSuccess && clusters > 0)
+    return Together::kCluster;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+      cudaFuncSetAttribute(mlp_train_steps_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           int(kTrainSmemBytes)) == cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_train_steps_kernel<false>, kTrainThreads,
+                                                    kTrainSmemBytes) == cudaSuccess &&
+      n_cta <= unsigned(sms) * unsigned(per_sm))
+    return Together::kCooperative;
+  cudaGetLastError();
+  return Together::kNo;
+}
+
+// Launch errors that say that the CTAs do not fit together here (a process limited to fewer SMs than the device has,
+// say); nothing was enqueued.
+bool does_not_fit(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+         e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidClusterSize;
 }
 
 cudaError_t train_tile_launch(const float* params, const float* x, int x_stride, const float* y, int y_stride,
@@ -849,7 +885,9 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
   const auto corrections = [&](uint32_t t) {
     return make_float2(1.0f - powf(beta1, float(t)), 1.0f - powf(beta2, float(t)));
   };
-  if (steps > 0 && steps < (uint64_t(1) << 32) && train_together(n_cta)) {  // many steps a launch
+  uint64_t done = 0;
+  Together how = steps < (uint64_t(1) << 32) ? train_together(n_cta) : Together::kNo;
+  if (how != Together::kNo) {  // many steps a launch
     TrainSteps a{};
     a.records = records;
     a.batch = batch;
@@ -862,51 +900,38 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
     a.epoch_loss = epoch_loss;
     a.q = sc.q;
     a.meet = sc.meet;
-    // 2, 4 or 8 CTAs (batches of 129 to 1024) as one cluster: its barrier takes a fifth of the counter's time
-    const bool cluster = n_cta == 2 || n_cta == 4 || n_cta == 8;
     a.lr = lr;
     a.beta1 = beta1;
     a.beta2 = beta2;
     a.eps = eps;
-    for (uint64_t done = 0; done < steps; done += a.count) {
+    while (done < steps) {
       a.first = uint32_t(done);
       a.count = uint32_t(steps - done < uint64_t(kTrainSteps) ? steps - done : uint64_t(kTrainSteps));
-      for (uint32_t i = 0; i < a.count; ++i) a.c[i] = corrections(++(*adam_t));
+      for (uint32_t i = 0; i < a.count; ++i) a.c[i] = corrections(*adam_t + i + 1);
       if ((e = cudaMemsetAsync(sc.meet, 0, sizeof(uint32_t), stream)) != cudaSuccess) return e;
-      cudaLaunchAttribute attr{};
-      if (cluster) {
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = n_cta;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-      } else {
-        attr.id = cudaLaunchAttributeCooperative;
-        attr.val.cooperative = 1;
+      const StepsConfig c(n_cta, how, stream);
+      e = how == Together::kCluster ? cudaLaunchKernelEx(&c.cfg, mlp_train_steps_kernel<true>, a)
+                                    : cudaLaunchKernelEx(&c.cfg, mlp_train_steps_kernel<false>, a);
+      if (does_not_fit(e)) {
+        cudaGetLastError();
+        break;
       }
-      cudaLaunchConfig_t cfg{};
-      cfg.gridDim = dim3(n_cta);
-      cfg.blockDim = dim3(kTrainThreads);
-      cfg.dynamicSmemBytes = kTrainSmemBytes;
-      cfg.stream = stream;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      e = cluster ? cudaLaunchKernelEx(&cfg, mlp_train_steps_kernel<true>, a)
-                  : cudaLaunchKernelEx(&cfg, mlp_train_steps_kernel<false>, a);
       if (e != cudaSuccess) return e;
+      *adam_t += a.count;
+      done += a.count;
     }
-    return cudaSuccess;
   }
-  for (uint32_t ep = 0; ep < epochs; ++ep) {
-    for (uint32_t b = 0; b < nb; ++b) {
-      const float* rec = records + size_t(b) * batch * kMlpRecord;
-      e = train_tile_launch(params, rec, kMlpRecord, rec + 12, kMlpRecord, batch, sc, stream);
-      if (e != cudaSuccess) return e;
-      const float2 c = corrections(++(*adam_t));
-      mlp_reduce_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(
-          sc.part, sc.sq, n_cta, 1.0f / float(batch), sc.grad, params, moments, moments + kMlpParams, lr, beta1, beta2,
-          eps, c.x, c.y, nullptr, epoch_loss + ep, 1.0f / float(nb));
-      e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
+  for (; done < steps; ++done) {  // one step in two launches
+    const float* rec = records + size_t(done % nb) * batch * kMlpRecord;
+    e = train_tile_launch(params, rec, kMlpRecord, rec + 12, kMlpRecord, batch, sc, stream);
+    if (e != cudaSuccess) return e;
+    const float2 c = corrections(*adam_t + 1);
+    mlp_reduce_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(
+        sc.part, sc.sq, n_cta, 1.0f / float(batch), sc.grad, params, moments, moments + kMlpParams, lr, beta1, beta2,
+        eps, c.x, c.y, nullptr, epoch_loss + done / nb, 1.0f / float(nb));
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    ++*adam_t;
   }
   return cudaSuccess;
 }
