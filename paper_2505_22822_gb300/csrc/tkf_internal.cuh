@@ -314,9 +314,10 @@ namespace tkf {
 size_t mlp_train_scratch_bytes(uint32_t batch);
 cudaError_t mlp_loss_grad(const float* params, const float* x, int x_stride, const float* y, int y_stride,
                           uint32_t n, float* grad, float* loss, void* scratch, cudaStream_t stream);
+// meet_polls: limit of the wait where a batch's CTAs meet by a counter; NaN parameters and losses when it runs out
 cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t epochs, float lr, float beta1,
                       float beta2, float eps, float* params, float* moments, uint32_t* adam_t, float* epoch_loss,
-                      void* scratch, cudaStream_t stream);
+                      void* scratch, cudaStream_t stream, uint32_t meet_polls = 1u << 22);
 cudaError_t mlp_forward(const float* params, const float* x, uint32_t n, float* out, cudaStream_t stream);
 cudaError_t mlp_init(float* params, uint64_t seed, cudaStream_t stream);
 size_t mlp_calibrate_scratch_bytes(uint32_t n);

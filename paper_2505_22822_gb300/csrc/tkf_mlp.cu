@@ -523,6 +523,7 @@ struct TrainSteps {
   float *p, *m, *v, *part, *sq, *epoch_loss;
   float* q;        // the parameters in the gradient's order, for the launch
   uint32_t* meet;  // arrivals of the grid barrier, zeroed before the launch
+  uint32_t meet_polls;  // limit of the counter's wait
   float lr, beta1, beta2, eps;
   float2 c[kTrainSteps];
 };
@@ -530,7 +531,7 @@ struct TrainSteps {
 // Every CTA of the launch arrives, then waits for the others: by the hardware barrier where the CTAs are
 // one cluster, else by a counter (bounded: false if the wait ran out).
 template <bool kCluster>
-__device__ bool train_meet(TrainSmem& sm, uint32_t* meet, uint32_t target) {
+__device__ bool train_meet(TrainSmem& sm, uint32_t* meet, uint32_t target, uint32_t polls) {
   if constexpr (kCluster) {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -541,12 +542,12 @@ __device__ bool train_meet(TrainSmem& sm, uint32_t* meet, uint32_t target) {
       __threadfence();
       atomicAdd(meet, 1u);
       uint32_t seen = 0, it = 0;
-      for (; it < (1u << 22); ++it) {
+      for (; it < polls; ++it) {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(meet) : "memory");
         if (int32_t(seen - target) >= 0) break;
         if (it > 4096) __nanosleep(100);
       }
-      sm.flag = it < (1u << 22);
+      sm.flag = it < polls;
       __threadfence();
     }
     __syncthreads();
@@ -581,20 +582,21 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const
     tile_records(a.records + size_t(step % a.batches) * a.batch * kMlpRecord, a.batch, rec);
   };
   load(a.first);
-  bool together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x));  // every slice of q is there
-  for (uint32_t i = 0; i < a.count && together; ++i) {
+  bool together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x), a.meet_polls);  // every slice of q is there
+  uint32_t i = 0;
+  for (; i < a.count && together; ++i) {
     train_weights<true>(sm, a.q);
     const TrainInput in = tile_input(sm, rec);
     if (ok) ok = train_tile(sm, tmem, phase, in, a.batch, inv_n, g, a.sq + blockIdx.x);
     if (!ok) train_failed(sm, phase, g, a.sq + blockIdx.x);
     if (i + 1 < a.count) load(a.first + i + 1);
-    together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x));
+    together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x), a.meet_polls);
     if (!together) break;
     if (blockIdx.x == 0 && threadIdx.x == kTrainThreads - 1) {
       float l = 0.0f;
       for (uint32_t c = 0; c < gridDim.x; ++c) l += __ldcg(a.sq + c);
       l *= inv_n;
-      a.epoch_loss[(a.first + i) / a.batches] += l * inv_batches;
+      atomicAdd(a.epoch_loss + (a.first + i) / a.batches, l * inv_batches);
     }
     const float2 c = a.c[i];
     // every element's sum runs over the CTAs in order; the loads of a thread's elements overlap
@@ -623,7 +625,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const
       reduce(std::integral_constant<int, 2>{});
     else
       reduce(std::integral_constant<int, kSliceMax>{});
-    together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x));
+    together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x), a.meet_polls);
   }
 #pragma unroll
   for (int q = 0; q < kSliceMax; ++q) {
@@ -635,6 +637,10 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const
       a.p[k] = together ? pk[q] : __int_as_float(0x7fc00000);
     }
   }
+  // a meeting that did not come about: with the parameters the losses of the epochs that it cut short are NaN
+  if (!together && threadIdx.x == 0)
+    for (uint32_t ep = (a.first + min(i, a.count - 1)) / a.batches; ep <= (a.first + a.count - 1) / a.batches; ++ep)
+      atomicExch(a.epoch_loss + ep, __int_as_float(0x7fc00000));
   train_teardown(tmem);
 }
 
@@ -875,7 +881,7 @@ cudaError_t mlp_loss_grad(const float* params, const float* x, int x_stride, con
 
 cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t epochs, float lr, float beta1,
                       float beta2, float eps, float* params, float* moments, uint32_t* adam_t, float* epoch_loss,
-                      void* scratch, cudaStream_t stream) {
+                      void* scratch, cudaStream_t stream, uint32_t meet_polls) {
   const TrainScratch sc = carve_train(scratch, batch);
   const uint32_t nb = n / batch;
   const unsigned n_cta = (batch + kTile - 1) / kTile;
@@ -900,6 +906,7 @@ cudaError_t mlp_train(const float* records, uint32_t n, uint32_t batch, uint32_t
     a.epoch_loss = epoch_loss;
     a.q = sc.q;
     a.meet = sc.meet;
+    a.meet_polls = meet_polls;
     a.lr = lr;
     a.beta1 = beta1;
     a.beta2 = beta2;
