@@ -63,7 +63,7 @@ __device__ __forceinline__ double rcp_nr(double x) {
   return fma(y, fma(e, e, e), y);
 }
 
-// 1/sqrt(x) of a normal x > 0, within about an ulp, in the same way.
+// 1/sqrt(x) of a normal x > 0, within 1.1 ulp, in the same way.
 __device__ __forceinline__ double rsqrt_nr(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -97,7 +97,10 @@ __device__ __forceinline__ void crossf(const double a[3], const double b[3], dou
 // Natural logarithm of a positive normal x (table-driven, after P. T. P. Tang, ACM TOMS 16, 1990):
 // x = 2^e m, c ~ 1/m from the top 7 bits of m, ln x = e ln 2 - ln c + ln(1 + z) with z = m c - 1,
 // |z| < 2^-8, by its series through z^7 (truncation below 2^-66). 11 FP64 instructions against about
-// 25 of log(); within 1.1 ulp in the callers' ranges (results of magnitude 4 to 40). Others: log().
+// 25 of log(). The sum with e ln 2 comes last, so that one rounding is of the result's size: within 1.1 ulp where its
+// magnitude is 4 to 40 (e times the rounding of ln 2, the table's and the small sum's 2^-53 in the rest), within 2^-50
+// below; with e ln 2 - ln c first and the series last, 1.31 ulp. The callers' results are of magnitude 0 to 40 (the
+// scattering's below 4 at steep incidence). Zero, negative, not normal: log().
 struct LogTable {
   double c[128], l[128];  // c, -ln c
 };
@@ -129,7 +132,7 @@ __device__ __forceinline__ double log_nr(double x) {
   p = fma(z, p, 1.0 / 3);
   p = fma(z, p, -0.5);
   p = fma(__dmul_rn(z, z), p, z);
-  return fma(f2d(float(e)), 0.693147180559945309417, __ldg(&kLogTable.l[j])) + p;
+  return fma(f2d(float(e)), 0.693147180559945309417, __ldg(&kLogTable.l[j]) + p);
 }
 
 // atan2(y, x) (table-driven, after P. T. P. Tang, ACM TOMS 16, 1990): with t = min / max of |x|, |y| and
