@@ -70,7 +70,7 @@ __device__ uint32_t helix_three_points(const double r1[3], const double r2[3], c
   out[0] = atan2_nr(ty, tx);
   out[1] = atan2_nr(arc, dz);
   sin_theta = arc * rsqrt_pos(arc * arc + dz * dz);
-  out[2] *= sin_theta;
+  if (st == 0) out[2] *= sin_theta;  // (sin(theta) of three equal points is NaN, their q/p 0)
   return st;
 }
 
