@@ -226,10 +226,10 @@ tkf_status tkf_geometry_create(tkf_context ctx, const tkf_surface_desc* s, uint3
   h->mat.log_hwp_over_i_f = float(h->mat.log_hwp_over_i);
   h->mat.bg2_density_f = float(h->mat.bg2_density);
   const double I = m.i_ev * 1e-9;
-  h->mat.two_me_over_i_sq = (2.0 * 0.51099895e-3 / I) * (2.0 * 0.51099895e-3 / I);
-  h->mat.dedx_scale = 0.307075 * m.z_over_a * m.rho_g_cm3 * 1e-4;
-  h->mat.two_me_over_i2_f = float(2.0 * 0.51099895e-3 / (I * I));
-  h->mat.dedx_scale_f = float(0.307075 * m.z_over_a * m.rho_g_cm3 * 1e-4);
+  h->mat.two_me_over_i_sq = (2.0 * tkf::kMe / I) * (2.0 * tkf::kMe / I);
+  h->mat.dedx_scale = tkf::kBetheK * m.z_over_a * m.rho_g_cm3 * 1e-4;
+  h->mat.two_me_over_i2_f = float(2.0 * tkf::kMe / (I * I));
+  h->mat.dedx_scale_f = float(tkf::kBetheK * m.z_over_a * m.rho_g_cm3 * 1e-4);
   *out = h;
   return TKF_OK;
 }
@@ -514,14 +514,14 @@ static tkf::FitArgs make_args(tkf_geometry geo, const tkf_fit_options* o, const 
   a.opt.surf_tol = o->surf_tol;
   a.opt.mass = o->mass;
   a.opt.inv_mass2 = 1.0 / (o->mass * o->mass);
-  a.opt.two_me_over_mass2 = 2.0 * 0.51099895e-3 / (o->mass * o->mass);
-  a.opt.one_me_mass2 = 1.0 + (0.51099895e-3 / o->mass) * (0.51099895e-3 / o->mass);
+  a.opt.two_me_over_mass2 = 2.0 * tkf::kMe / (o->mass * o->mass);
+  a.opt.one_me_mass2 = 1.0 + (tkf::kMe / o->mass) * (tkf::kMe / o->mass);
   a.opt.max_steps = o->max_steps;
   a.opt.tol_f = float(o->tol);
   a.opt.h_max_f = float(o->h_max);
   a.opt.h_min_f = float(o->h_min);
   a.opt.mass_f = float(o->mass);
-  a.opt.me_over_mass_f = float(0.51099895e-3 / o->mass);
+  a.opt.me_over_mass_f = float(tkf::kMe / o->mass);
   a.opt.surf_tol_f = float(o->surf_tol);
   a.mlp = (o->step_mode == TKF_STEP_LEARNED && o->mlp) ? o->mlp->d_weights : nullptr;
   a.records = (o->step_mode == TKF_STEP_ADAPTIVE) ? o->records : nullptr;

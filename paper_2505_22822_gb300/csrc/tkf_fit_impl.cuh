@@ -30,8 +30,6 @@ namespace tkf {
 namespace {
 
 constexpr double kKappa = 2.99792458e-4;  // GeV / (T mm)
-constexpr double kMe = 0.51099895e-3;  // GeV
-constexpr double kBetheK = 0.307075;   // MeV cm^2 / mol
 
 constexpr uint32_t kFatal = ~(TKF_TRACK_TOO_FEW_HITS | TKF_TRACK_OUT_OF_FIELD | TKF_TRACK_PROPOSAL_FALLBACK);
 

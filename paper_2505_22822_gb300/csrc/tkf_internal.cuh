@@ -21,9 +21,12 @@ namespace tkf {
 //   the navigation's screens), 2 x 0.
 constexpr int kSurfStride = 24;
 
+constexpr double kMe = 0.51099895e-3;  // electron mass, GeV
+constexpr double kBetheK = 0.307075;   // MeV cm^2 / mol
+
 // Material constants folded for the kernels.
 struct MaterialDev {
-  double z_over_a, i_ev, rho, hwp_ev;
+  double z_over_a, i_ev, rho, hwp_ev;  // as given: for the graph's key, read by no kernel
   double log_hwp_over_i;  // ln(hbar omega_p / I)
   double bg2_density;     // (beta gamma)^2 above which the density-effect term is positive
   double two_me_over_i_sq;  // (2 m_e / I)^2
