@@ -583,7 +583,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const
   };
   load(a.first);
   bool together = train_meet<kCluster>(sm, a.meet, (met += gridDim.x), a.meet_polls);  // every slice of q is there
-  uint32_t i = 0;
+  uint32_t i = 0, epoch = a.first / a.batches;  // the current epoch and its loss so far (one thread's)
+  float sum = __ldcg(a.epoch_loss + epoch);
   for (; i < a.count && together; ++i) {
     train_weights<true>(sm, a.q);
     const TrainInput in = tile_input(sm, rec);
@@ -596,7 +597,14 @@ __global__ void __launch_bounds__(kTrainThreads, 1) mlp_train_steps_kernel(const
       float l = 0.0f;
       for (uint32_t c = 0; c < gridDim.x; ++c) l += __ldcg(a.sq + c);
       l *= inv_n;
-      atomicAdd(a.epoch_loss + (a.first + i) / a.batches, l * inv_batches);
+      if ((a.first + i) / a.batches != epoch) {
+        ++epoch;
+        sum = 0.0f;
+      }
+      // stored by comparison: not over the NaN that a CTA left whose meeting failed
+      const float next = fmaf(l, inv_batches, sum);
+      atomicCAS(reinterpret_cast<unsigned*>(a.epoch_loss + epoch), __float_as_uint(sum), __float_as_uint(next));
+      sum = next;
     }
     const float2 c = a.c[i];
     // every element's sum runs over the CTAs in order; the loads of a thread's elements overlap
