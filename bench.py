@@ -46,8 +46,9 @@ WORKLOAD_MAP = "solenoid_map_100k_muons"
 # in R = P J^T (45 flops fewer per propagated measurement).
 FLOPS = {
     "fp64": (493, 111, 1494, 330),
-    # the FP64 path in a field along z: closed-form steps (34 an attempt; the "fp64" rows are the
-    # stage-by-stage form of any other field)
+    # the FP64 path in a field along z: closed-form steps (34 an attempt). The "fp64" rows are the
+    # stage-by-stage form as it was captured below; any other field takes that form, which now
+    # shares T x B between the state and the q/p column: (424, 125, 1481, 330)
     "fp64_axial": (103, 41, 1168, 330),
     "fp64_axial_two_filter": (103, 41, 1617, 1837),
     # mixed: only the FP64 anchors, the Joseph update and the smoother count
@@ -60,13 +61,15 @@ FLOPS = {
 }
 # r-z field map: every attempt adds two stage positions and three bilinear lookups (FP64 in
 # the plain path: 32 flops each incl. one square root and one division), every propagated
-# measurement two more lookups; the mixed path looks up in FP32.
+# measurement two more lookups; the mixed path looks up in FP32. FP64: T x B is formed once a
+# stage for the state and the q/p column (an attempt +14, an accepted step's columns -83, +6 for the
+# field at three places), a landing takes 3 fewer, the material, whose constants are folded, 11.
 FLOPS_MAP = {
-    "fp64": (619, 237, 1558, 330),
+    "fp64": (556, 251, 1545, 330),
     "mixed": (20, 8, 749, 330),
     "mixed_learned": (20, 8, 749, 330),
     "mixed_fp32": (20, 8, 45, 30),
-    "fp64_two_filter": (619, 237, 2337, 1837),
+    "fp64_two_filter": (556, 251, 2311, 1837),
     "mixed_two_filter": (20, 8, 722, 1837),
 }
 
@@ -79,19 +82,22 @@ FLOPS_MAP = {
 # launch and are scaled by tracks to a full launch. Keyed by (workload, variant, register cap of
 # the launched kernel); a kernel change voids the entries (profiles/ keeps the commands).
 CAPTURES = {
-    ("barrel", "mixed_learned", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5100021,
-        "rejected": 17506, "shape": "128,4,32,128", "dram_bytes": 1495617024,
-        "fp64_exec": 2357505588, "fp64_model": 2281033040, "fp32_exec": 3651469626},
+    ("barrel", "mixed_learned", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5104781,
+        "rejected": 23922, "shape": "128,4,32,128", "dram_bytes": 1526147584,
+        "fp64_exec": 2370174320, "fp64_model": 2281051248, "fp32_exec": 3572956959},
+    # (before the update divided and the sums of two products had a fixed order; since then DRAM 1473998080,
+    # FP64 2367389840, FP32 3526630696)
     ("barrel", "mixed", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014959,
         "rejected": 143605, "shape": "128,4,32,128", "dram_bytes": 1458471424,
         "fp64_exec": 2354693398, "fp64_model": 2277818612, "fp32_exec": 3604152818},
     ("barrel", "fp64_axial", 255): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014958,
-        "rejected": 143611, "shape": "128,2,32,255", "dram_bytes": 1047469568,
+        "rejected": 143611, "shape": "128,2,32,255", "dram_bytes": 1047698944,
         "fp64_exec": 4627625879, "fp64_model": 4062418156, "fp32_exec": 207284986},
     ("barrel", "fp64_axial", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014958,
-        "rejected": 143611, "shape": "128,4,32,128", "dram_bytes": 2143469056,
+        "rejected": 143611, "shape": "128,4,32,128", "dram_bytes": 2138513120,
         "fp64_exec": 4645413017, "fp64_model": 4062418156, "fp32_exec": 234135716},
-    # the stage-by-stage form, which the FP64 path took on this batch before the closed-form steps
+    # the stage-by-stage form as the FP64 path took it on this batch before the closed-form steps: no
+    # launch of this benchmark runs it, it is the measure of what those steps and the mixed path save
     ("barrel", "fp64", 128): {"tracks": 279450, "hits_after_first": 2964523, "attempts": 5014958, "rejected": 143611,
                               "shape": "128,4,32,128", "dram_bytes": 2871720960,
                               "fp64_exec": 8183930686, "fp64_model": 6938730754, "fp32_exec": 71595040},

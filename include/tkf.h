@@ -587,7 +587,8 @@ typedef struct tkf_mlp_train_options {
  * records [n][TKF_MLP_RECORD] (inputs, label), params [TKF_MLP_PARAMS], adam_moments
  * [2][TKF_MLP_PARAMS] (first and second moments; zero them before the first call),
  * epoch_loss [epochs] (mean loss of each epoch). *adam_t (HOST) counts the Adam steps taken so
- * far (0 before the first call) and is advanced. Scratch comes from the context workspace.
+ * far (0 before the first call) and is advanced by the steps enqueued. Scratch comes from the context
+ * workspace. A wait on the device that runs out (they are bounded) leaves NaN parameters and losses.
  * Errors: TKF_ERR_INVALID_ARG (NULL, batch out of range or larger than n), TKF_ERR_OOM,
  * TKF_ERR_DEVICE. */
 tkf_status tkf_mlp_train(tkf_context ctx, const float* records, uint32_t n, const tkf_mlp_train_options* opts,

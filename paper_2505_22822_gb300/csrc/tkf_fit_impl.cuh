@@ -2127,8 +2127,9 @@ __global__ void __launch_bounds__(reg_block_threads(kRegs), reg_min_blocks(kRegs
                           uint32_t tpw) {
   constexpr int kPlace = kPrec == 2 ? 0 : reg_state_place(kRegs);
   // the column loops stay rolled at 64 registers, and out of step in the mixed path's field map at 128 too, whose
-  // code is the longest (three lookups a step; 100,000 map muons 1.39 -> 1.36 ms); in step the unrolled loops
-  // are as fast or faster (100,000 1.30 -> 1.25, two-filter 200,000 3.39 -> 3.27)
+  // code is the longest (three lookups a step): of the present kernels the all-states fit with that cap (measured on the
+  // plain fit when it was out of step: 100,000 map muons 1.39 -> 1.36 ms). In step the unrolled loops are as fast
+  // or faster (100,000 1.30 -> 1.25, two-filter 200,000 3.39 -> 3.27)
   constexpr bool kRoll =
       kRegs == 64 || (kRegs == 128 && kPrec == 1 && !F::kUniform && !in_step(kPrec, kMode, kRegs, kG));
   extern __shared__ double smem_state[];

@@ -37,7 +37,9 @@ __device__ __forceinline__ float d2f(double x) {
 // instructions: 1 to 4). The FP64 path's stepping therefore takes reciprocals and roots by
 // Newton-Raphson (or one third-order step, which cubes the relative error) from the special-function
 // unit's or an FP32 seed, and compares magnitudes as integers. Products that feed a sum are written
-// as fma() or __dmul_rn, so that every instantiation (register caps, lanes a track) rounds alike.
+// as fma() or __dmul_rn, or as mul_add and mul_sub below, so that they round alike in every instantiation (register
+// caps, lanes a track). Sums of the FP64 path's general code that are left to the compiler have rounded alike in all of
+// them so far (tilted and axial fields, the map), which nothing guarantees.
 
 // |x| <= lim and |x| < lim for lim >= 0: the bit patterns of non-negative doubles order like the
 // values, NaN above all (so a NaN x is neither).

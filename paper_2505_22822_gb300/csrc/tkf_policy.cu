@@ -1,8 +1,9 @@
 // tkf_policy.cu -- launch policy of the fit: launch-shape autotuning and CUDA-graph replay.
 //
 // Neither changes what a track computes: every thread fits its own tracks with the same
-// arithmetic whatever the launch shape, and a graph replays exactly the launches that a
-// direct call makes.
+// operations whatever the launch shape (the mixed fit to the bit; FP64 kernels of other register
+// caps are other instantiations, whose general code the compiler could fuse differently), and a
+// graph replays exactly the launches that a direct call makes.
 
 #include <errno.h>
 #include <math.h>
